@@ -223,6 +223,8 @@ struct __align__(16) DgChemMlp {
   double tol_check, floor;
 };
 
+constexpr int CHEM_NR = 1;  // rows per thread of the tile engine (the decode needs the registers)
+
 __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
   x += 0x9E3779B97F4A7C15ull;
   x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -257,20 +259,21 @@ __device__ __forceinline__ void chem_features(const T* uu, int np, double Tk, fl
 // cmode 2 (refresh): only the decoded rates (jpi' before its clamp) are written to corr,
 // for chem_refresh_kernel to turn into corrections.
 template <typename T>
-__global__ void __launch_bounds__(dgtc5::THREADS, 1)
+__global__ void __launch_bounds__(dgtc5::THREADS, 4)
 chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, const DgChemMlp* mlp,
                     const double* dtp, T* src, unsigned char* flags, float* corr, const unsigned char* trust,
                     int cmode) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  dgtc5::Smem<10>& s = *reinterpret_cast<dgtc5::Smem<10>*>(smem_raw);
+  dgtc5::Smem<10, CHEM_NR>& s = *reinterpret_cast<dgtc5::Smem<10, CHEM_NR>*>(smem_raw);
+  dgtc5::alloc_tmem<10, CHEM_NR>(s);
   __shared__ DgChemMlp m;
   dgmlp::copy_to_smem(m, mlp);
   __syncthreads();
-  dgtc5::load_weights<10>(s, m.w);
+  dgtc5::load_weights<10, CHEM_NR>(s, m.w);
   const int nv = NSPEC + dim + 1;
   const int64_t total = K * np;
   const float dt = dtp ? (float)*dtp : 0.f;
-  auto prod = [&](int64_t i, float* x) {
+  auto prod = [&](int64_t i, float* x, int) {
     float raw[7];
     bool ok = true;
     if (i < total) {
@@ -286,7 +289,7 @@ chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, co
     x[7] = 0.f;
     return ok;
   };
-  auto cons = [&](int64_t i, const float* y, bool ok, bool valid) {
+  auto cons = [&](int64_t i, const float* y, bool ok, bool valid, int) {
     if (cmode == 2) {  // uniform over the grid: no lane reaches the vote below
       if (i < total && valid) {
 #pragma unroll
@@ -334,7 +337,7 @@ chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, co
       flags[base >> 5] = !trusted ? 4 : (tile_ok ? 0 : 1);
     }
   };
-  dgtc5::run_tiles<10>(s, total, prod, cons);
+  dgtc5::run_tiles<10, CHEM_NR>(s, total, prod, cons);
 }
 
 // one thread per tile still accepted: compare the learned source at the tile's sampled
@@ -558,14 +561,13 @@ template <typename T>
 static cudaError_t chem_learned(DgThermo* th, const T* u, const double* dt_dev, int refresh, cudaStream_t s) {
   const int64_t total = th->K * th->np, ntiles = (total + 31) / 32;
   const DgChemMlp* m = (const DgChemMlp*)th->chem_mlp;
-  // tensor-core tiles of 128 nodes; the dynamic shared memory is padded to 60 KB so that at
-  // most 3 CTAs (3 x 128 tensor-memory columns) share an SM
-  const size_t smem = sizeof(dgtc5::Smem<10>) > 60 * 1024 ? sizeof(dgtc5::Smem<10>) : 60 * 1024;
+  // persistent CTAs over tensor-core tiles of 128 nodes
+  const size_t smem = sizeof(dgtc5::Smem<10, CHEM_NR>);
   auto k1 = chem_mlp_tc5_kernel<T>;
   cudaError_t e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int64_t t128 = (total + dgtc5::ROWS - 1) / dgtc5::ROWS;
-  const unsigned g1 = (unsigned)(t128 < 152 * 3 ? t128 : 152 * 3);
+  const unsigned g1 = (unsigned)(t128 < 152 * 4 ? t128 : 152 * 4);
   if (refresh) {
     if (!th->chem_corr || !th->chem_trust) return cudaErrorInvalidValue;
     k1<<<g1, dgtc5::THREADS, smem, s>>>(u, th->T, th->K, th->np, th->dim, m, dt_dev, (T*)th->src,

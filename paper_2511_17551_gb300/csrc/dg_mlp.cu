@@ -70,20 +70,21 @@ __device__ __forceinline__ double clampT(double T) { return T < 200.0 ? 200.0 : 
 // predicted temperature by one Newton step with the residual check, or runs the plain
 // Newton iteration (fallback, counted; also when the engine's waits ran out).
 template <typename T>
-__global__ void __launch_bounds__(dgtc5::THREADS, 1)
+__global__ void __launch_bounds__(dgtc5::THREADS, 4)
 thermo_mlp_kernel(const T* u, int64_t K, int np, int dim, const double* sp, const float* sp32, double* Tc,
                   T* pc, unsigned long long* status, const DgMlpDev* mlp, unsigned long long* stats) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  dgtc5::Smem<1>& sm = *reinterpret_cast<dgtc5::Smem<1>*>(smem_raw);
+  dgtc5::Smem<1, 1>& sm = *reinterpret_cast<dgtc5::Smem<1, 1>*>(smem_raw);
+  dgtc5::alloc_tmem<1, 1>(sm);
   __shared__ DgMlpDev m;
   copy_to_smem(m, mlp);
   __syncthreads();
-  dgtc5::load_weights<1>(sm, m.w);
+  dgtc5::load_weights<1, 1>(sm, m.w);
   const int nv = NSPEC + dim + 1;
   const int64_t total = K * np;
   unsigned long long n_ok = 0, n_fb = 0;
   double Y[NSPEC], rho = 1.0, e = 0.0;  // this thread's node, carried from features to polish
-  auto prod = [&](int64_t i, float* x) {
+  auto prod = [&](int64_t i, float* x, int) {
     if (i < total) {
       const T* uu = u + (i / np) * nv * np + (i % np);
       rho = 0.0;
@@ -127,7 +128,7 @@ thermo_mlp_kernel(const T* u, int64_t K, int np, int dim, const double* sp, cons
     }
     return false;
   };
-  auto cons = [&](int64_t i, const float* y, bool, bool valid) {
+  auto cons = [&](int64_t i, const float* y, bool, bool valid, int) {
     if (i >= total) return;
     const int64_t k = i / np;
     const int node = (int)(i % np);
@@ -200,7 +201,7 @@ thermo_mlp_kernel(const T* u, int64_t K, int np, int dim, const double* sp, cons
       pc[(k * 2 + 1) * np + node] = (T)sqrt((cv + P.Rmix) / cv * p / rho);
     }
   };
-  dgtc5::run_tiles<1>(sm, total, prod, cons);
+  dgtc5::run_tiles<1, 1>(sm, total, prod, cons);
   if (stats) {
     for (int o = 16; o > 0; o >>= 1) {
       n_ok += __shfl_xor_sync(0xffffffffu, n_ok, o);
@@ -472,11 +473,10 @@ cudaError_t dg_mlp_set(DgThermo* th, const float* params_host, const double* sta
 
 cudaError_t dg_mlp_thermo_update(DgThermo* th, const void* u, int f32, cudaStream_t s) {
   const int64_t n = th->K * th->np;
-  // tensor-core tiles of 128 nodes; the dynamic shared memory is padded to 60 KB so that at
-  // most 3 CTAs (3 x 128 tensor-memory columns) share an SM
-  const size_t smem = sizeof(dgtc5::Smem<1>) > 60 * 1024 ? sizeof(dgtc5::Smem<1>) : 60 * 1024;
+  // persistent CTAs over tensor-core tiles of 128 nodes
+  const size_t smem = sizeof(dgtc5::Smem<1, 1>);
   const int64_t t128 = (n + dgtc5::ROWS - 1) / dgtc5::ROWS;
-  const unsigned grid = (unsigned)(t128 < 152 * 3 ? t128 : 152 * 3);
+  const unsigned grid = (unsigned)(t128 < 152 * 4 ? t128 : 152 * 4);
   cudaError_t e;
   if (f32) {
     auto k = thermo_mlp_kernel<float>;
@@ -506,22 +506,23 @@ cudaError_t dg_mlp_sample(DgThermo* th, const void* u, int f32, int64_t n, uint6
   return cudaGetLastError();
 }
 
-// tcgen05 forward: persistent CTAs of 128 threads over 128-row tiles; the dynamic
-// shared memory is padded to 60 KB so that at most 3 CTAs (3 x 128 tensor-memory columns)
-// share an SM
+// tcgen05 forward: persistent CTAs of 128 threads over 256-row tiles
 __device__ unsigned g_tc5_err;
 template <int NO>
 static dg_status forward_tc5(const float* P, const float* X, float* y, int64_t n, cudaStream_t st) {
-  const size_t smem = sizeof(dgtc5::Smem<NO>) > 60 * 1024 ? sizeof(dgtc5::Smem<NO>) : 60 * 1024;
+  const size_t smem = sizeof(dgtc5::Smem<NO, dgtc5::FWD_NR>);
   auto k = dgtc5::mlp_forward_tc5_kernel<NO>;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess)
     return DG_ECUDA;
   unsigned* err = NULL;
   if (cudaGetSymbolAddress((void**)&err, g_tc5_err) != cudaSuccess) return DG_ECUDA;
   if (cudaMemsetAsync(err, 0, sizeof(unsigned), st) != cudaSuccess) return DG_ECUDA;
-  const int64_t tiles = (n + dgtc5::ROWS - 1) / dgtc5::ROWS;
-  const unsigned grid = (unsigned)(tiles < 152 * 3 ? tiles : 152 * 3);
-  k<<<grid, dgtc5::THREADS, smem, st>>>(P, X, y, n, err);
+  const int64_t rows = dgtc5::FWD_NR * dgtc5::ROWS, tiles = (n + rows - 1) / rows;
+  const int64_t ctas = 152 * 2 * dgtc5::FWD_CTAS;  // two waves of resident CTAs: 339 against 350 us at 4.6 M rows
+  const unsigned grid = (unsigned)(tiles < ctas ? tiles : ctas);
+  const int vec = (((uintptr_t)X | (uintptr_t)y) & 15) == 0;
+  k<<<grid, dgtc5::THREADS, smem, st>>>(P, X, y, n, err, vec);
   if (cudaGetLastError() != cudaSuccess) return DG_ECUDA;
   unsigned h = 0;
   if (cudaMemcpyAsync(&h, err, sizeof(unsigned), cudaMemcpyDeviceToHost, st) != cudaSuccess) return DG_ECUDA;
