@@ -12,12 +12,13 @@
 // T <- T - (e(T) - e)/cv(T) is warm-started from the node's previous temperature and
 // stops at |dT| <= 1e-12 T (at most 50 steps, T kept in [200, 1e4] K); failure latches
 // DG_ENEWTON.  Mixed form: FP32 Newton on e(T) - b0 = e - b0 (the constant b0 is
-// removed so FP32 resolves the residual) to |dT| <= 1e-6 T, then FP64 Newton steps on
-// the FP64 residual (normally one).
+// removed so FP32 resolves the residual) to |dT| <= 1e-6 T, then one Newton step on the
+// residual in double-FP32 pairs.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
 
+#include "dg_dd.cuh"
 #include "dg_internal.h"
 #include "dg_thermo.h"
 
@@ -72,80 +73,30 @@ __device__ __forceinline__ bool newton64(const Poly<double>& P, double e, double
   return false;
 }
 
-template <typename T>
-__global__ void thermo_update_kernel(const T* u, int64_t K, int np, int dim, const double* cf,
-                                     const float* cf32, double* Tc, T* pc,
-                                     unsigned long long* status, int mixed) {
+// FP64 form: the full FP64 Newton iteration, one thread per node
+__global__ void thermo_update_kernel(const double* u, int64_t K, int np, int dim, const double* cf, double* Tc,
+                                     double* pc, unsigned long long* status) {
   const int nv = NSPEC + dim + 1;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < K * np;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t k = i / np;
     const int node = (int)(i % np);
-    const T* uu = u + k * nv * np + node;
+    const double* uu = u + k * nv * np + node;
     double Y[NSPEC], rho = 0.0, ke = 0.0;
 #pragma unroll
     for (int s = 0; s < NSPEC; ++s) {
-      Y[s] = (double)uu[s * np];
+      Y[s] = uu[s * np];
       rho += Y[s];
     }
     for (int d = 0; d < dim; ++d) {
-      const double m = (double)uu[(NSPEC + d) * np];
+      const double m = uu[(NSPEC + d) * np];
       ke += m * m;
     }
     const double ir = 1.0 / rho;
-    const double e = (double)uu[(NSPEC + dim) * np] * ir - 0.5 * ke * ir * ir;
+    const double e = uu[(NSPEC + dim) * np] * ir - 0.5 * ke * ir * ir;
     double Tk = Tc[k * np + node];
     if (!(Tk >= 200.0 && Tk <= 1e4)) Tk = 1000.0;
     Poly<double> P;
-    if (mixed) {
-      // FP32 mixture polynomial for the Newton iteration; in FP64 only the large constant
-      // b0 (formation energies), from density-weighted sums
-      Poly<float> Pf;
-      float Yf[NSPEC];
-      double b0 = 0.0;
-      const float irf = (float)ir;
-#pragma unroll
-      for (int s = 0; s < NSPEC; ++s) {
-        Yf[s] = (float)Y[s] * irf;
-        b0 += Y[s] * cf[8 * s];
-      }
-      b0 *= ir;
-      build_poly<float>(cf32, Yf, Pf);
-      const float er = (float)(e - b0);
-      float Tf = (float)Tk;
-      bool conv = false;
-      for (int it = 0; it < 12; ++it) {
-        const float Tn = clampTf(Tf - (Pf.e_noconst(Tf) - er) / Pf.cv(Tf));
-        const float step = fabsf(Tn - Tf);
-        Tf = Tn;
-        if (step <= 1e-6f * Tf) {
-          conv = true;
-          break;
-        }
-      }
-      // the FP64 final residual: one Newton correction on e64(T) - e, evaluated in FP64
-      // with the FP64 constant b0 and the FP32-rounded temperature coefficients (their
-      // rounding moves e by ~1e-7 relative, i.e. T by ~1e-4 K); cv in FP32 only scales the
-      // correction.  The full FP64 iteration runs only where the FP32 stage did not converge.
-      double T64 = (double)Tf;
-      const double r = (b0 + T64 * ((double)Pf.b[1] + T64 * ((double)Pf.b[2] + T64 * ((double)Pf.b[3] +
-                        T64 * ((double)Pf.b[4] + T64 * (double)Pf.b[5]))))) - e;
-      T64 = clampT(T64 - r * (double)(1.0f / Pf.cv(Tf)));
-      bool ok = rho > 0.0;
-      if (ok && !conv) {
-#pragma unroll
-        for (int s = 0; s < NSPEC; ++s) Y[s] *= ir;
-        build_poly<double>(cf, Y, P);
-        ok = newton64(P, e, T64);
-      }
-      if (!ok) latch(status, DG_ST_NEWTON, k);
-      Tc[k * np + node] = T64;
-      const float Tq = (float)T64, rhof = (float)rho;
-      const float pf = rhof * Pf.Rmix * Tq, cvf = Pf.cv(Tq);
-      pc[(k * 2 + 0) * np + node] = (T)pf;
-      pc[(k * 2 + 1) * np + node] = (T)sqrtf((cvf + Pf.Rmix) / cvf * pf / rhof);
-      continue;
-    }
 #pragma unroll
     for (int s = 0; s < NSPEC; ++s) Y[s] *= ir;
     build_poly<double>(cf, Y, P);
@@ -154,8 +105,114 @@ __global__ void thermo_update_kernel(const T* u, int64_t K, int np, int dim, con
     Tc[k * np + node] = Tk;
     const double p = rho * P.Rmix * Tk;
     const double cv = P.cv(Tk);
-    pc[(k * 2 + 0) * np + node] = (T)p;
-    pc[(k * 2 + 1) * np + node] = (T)sqrt((cv + P.Rmix) / cv * p * ir);
+    pc[(k * 2 + 0) * np + node] = p;
+    pc[(k * 2 + 1) * np + node] = sqrt((cv + P.Rmix) / cv * p * ir);
+  }
+}
+
+// the full FP64 iteration of a mixed-form node whose FP32 iteration did not converge, from T
+__device__ __noinline__ bool newton64_node(const float* uu, int np, int dim, const double* cf, double& T) {
+  double Y[NSPEC], rho = 0.0, ke = 0.0;
+  for (int s = 0; s < NSPEC; ++s) {
+    Y[s] = (double)uu[s * np];
+    rho += Y[s];
+  }
+  for (int d = 0; d < dim; ++d) {
+    const double m = (double)uu[(NSPEC + d) * np];
+    ke += m * m;
+  }
+  const double ir = 1.0 / rho;
+  for (int s = 0; s < NSPEC; ++s) Y[s] *= ir;
+  Poly<double> P;
+  build_poly<double>(cf, Y, P);
+  return newton64(P, (double)uu[(NSPEC + dim) * np] * ir - 0.5 * ke * ir * ir, T);
+}
+
+// Mixed form: FP32 Newton on e(T) - b0 = e - b0, then one Newton correction on a residual in
+// double-FP32 pairs (dg_dd.cuh): the FP32 state is exact in them, e - b0 keeps 46 bits through
+// the cancellation of the formation energies, and the polynomial takes the FP32-rounded
+// temperature coefficients (their rounding moves e by ~1e-7 relative, i.e. T by ~1e-4 K, as it
+// did with the residual in FP64).  Nothing in the common path touches the FP64 pipe but the
+// conversions of the cached temperature; 68 FP64 instructions a node bound the kernel before.
+// Bytes per node: 36 of state, 16 of T, 8 of (p, c).  1.73 M nodes: 193 -> 55 us (1.9 TB/s), 4.6 M:
+// 500 -> 113 us (2.4 TB/s); the same distance to the FP64 solution (1.6e-7, the coefficients').
+template <int NP, int DIM>
+__global__ void __launch_bounds__(256, 3) thermo_mixed_kernel(const float* u, int64_t K, const double* cf,
+                                                           const float* cf32, double* Tc, float* pc,
+                                                           unsigned long long* status) {
+  using namespace dgdd;
+  constexpr int NV = NSPEC + DIM + 1;
+  __shared__ __align__(16) float c32[8 * NSPEC];
+  __shared__ dd b0s[NSPEC];
+  if (threadIdx.x < 8 * NSPEC) c32[threadIdx.x] = cf32[threadIdx.x];
+  if (threadIdx.x < NSPEC) b0s[threadIdx.x] = from_double(cf[8 * threadIdx.x]);
+  __syncthreads();
+  for (int64_t base = blockIdx.x * (int64_t)256; base < K * NP; base += gridDim.x * (int64_t)256) {
+    // element and node of base + threadIdx.x: the 64-bit division is the same in all threads
+    const int64_t k0 = base / NP;
+    const int off = (int)(base - k0 * NP) + (int)threadIdx.x;
+    const int64_t k = k0 + off / NP;
+    const int node = off % NP;
+    if (k >= K) continue;
+    const float* uu = u + k * NV * NP + node;
+    float r[NSPEC], m[DIM];
+#pragma unroll
+    for (int s = 0; s < NSPEC; ++s) r[s] = uu[s * NP];
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) m[d] = uu[(NSPEC + d) * NP];
+    const float E = uu[(NSPEC + DIM) * NP];
+    double Tk = Tc[k * NP + node];
+    dd rho = make(r[0], 0.f), ke = make(0.f, 0.f), b0 = mul(b0s[0], r[0]);
+#pragma unroll
+    for (int s = 1; s < NSPEC; ++s) {
+      acc(rho, make(r[s], 0.f));
+      acc_mul(b0, b0s[s], r[s]);
+    }
+    rho = norm(rho);
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) acc(ke, two_prod(m[d], m[d]));
+    const dd ir = rcp(rho);
+    // rho (e - b0) = E - |m|^2 / (2 rho) - sum rho_s b0_s
+    dd er = mul(mul(norm(ke), ir), -0.5f);
+    acc(er, make(E, 0.f));
+    acc(er, neg(b0));
+    er = mul(norm(er), ir);
+    Poly<float> P;
+    float Y[NSPEC];
+#pragma unroll
+    for (int s = 0; s < NSPEC; ++s) Y[s] = r[s] * ir.h;
+    build_poly<float>(c32, Y, P);
+    if (!(Tk >= 200.0 && Tk <= 1e4)) Tk = 1000.0;
+    float Tf = (float)Tk;
+    bool conv = false;
+    // (below 1e-12 kg/m^3 the products' low parts leave FP32's range: FP64)
+    for (int it = 0; it < 12 && rho.h > 1e-12f; ++it) {
+      const float Tn = clampTf(Tf - (P.e_noconst(Tf) - er.h) / P.cv(Tf));
+      const float step = fabsf(Tn - Tf);
+      Tf = Tn;
+      if (step <= 1e-6f * Tf) {
+        conv = true;
+        break;
+      }
+    }
+    // residual at Tf (exact in FP32) and the correction; cv in FP32 only scales it
+    dd q = add(two_prod(P.b[5], Tf), P.b[4]);
+    q = add(mul(q, Tf), P.b[3]);
+    q = add(mul(q, Tf), P.b[2]);
+    q = add(mul(q, Tf), P.b[1]);
+    q = add(mul(q, Tf), neg(er));
+    dd T = two_sum(Tf, -(q.h * (1.0f / P.cv(Tf))));
+    if (T.h < 200.f || (T.h == 200.f && T.l < 0.f)) T = make(200.f, 0.f);
+    if (T.h > 1e4f || (T.h == 1e4f && T.l > 0.f)) T = make(1e4f, 0.f);
+    double T64 = to_double(T);
+    bool ok = rho.h > 0.f;
+    if (ok && !conv) ok = newton64_node(uu, NP, DIM, cf, T64);
+    if (!ok) latch(status, DG_ST_NEWTON, k);
+    Tc[k * NP + node] = T64;
+    const float Tq = (ok && !conv) ? (float)T64 : T.h;
+    const float pf = rho.h * P.Rmix * Tq, cvf = P.cv(Tq);
+    pc[(k * 2 + 0) * NP + node] = pf;
+    pc[(k * 2 + 1) * NP + node] = sqrtf((cvf + P.Rmix) / cvf * pf / rho.h);
   }
 }
 
@@ -281,14 +338,18 @@ cudaError_t dg_thermo_reset(DgThermo* th, cudaStream_t s) {
 
 cudaError_t dg_thermo_update(DgThermo* th, const void* u, int f32, cudaStream_t s) {
   if (th->mode == 1 && th->mlp) return dg_mlp_thermo_update(th, u, f32, s);
-  if (f32)
-    thermo_update_kernel<float><<<grid_of(th->K * th->np), 256, 0, s>>>(
-        (const float*)u, th->K, th->np, th->dim, th->species, th->coef32, th->T, (float*)th->pc,
-        th->status, 1);
-  else
-    thermo_update_kernel<double><<<grid_of(th->K * th->np), 256, 0, s>>>(
-        (const double*)u, th->K, th->np, th->dim, th->species, th->coef32, th->T,
-        (double*)th->pc, th->status, 0);
+  if (!f32) {
+    thermo_update_kernel<<<grid_of(th->K * th->np), 256, 0, s>>>((const double*)u, th->K, th->np, th->dim, th->species,
+                                                                 th->T, (double*)th->pc, th->status);
+  } else if (th->dim == 3 && th->np == 64) {
+    thermo_mixed_kernel<64, 3><<<grid_of(th->K * th->np), 256, 0, s>>>((const float*)u, th->K, th->species, th->coef32,
+                                                                       th->T, (float*)th->pc, th->status);
+  } else if (th->dim == 3 && th->np == 125) {
+    thermo_mixed_kernel<125, 3><<<grid_of(th->K * th->np), 256, 0, s>>>((const float*)u, th->K, th->species, th->coef32,
+                                                                        th->T, (float*)th->pc, th->status);
+  } else {
+    return cudaErrorInvalidValue;  // mixtures are 3D with N = 3 or 4
+  }
   return cudaGetLastError();
 }
 
