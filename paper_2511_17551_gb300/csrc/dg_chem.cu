@@ -1,5 +1,7 @@
 // Finite-rate chemistry source on the device (appendix, Chemical Kinetics: Eqs. nrp,
-// forward_rate, backward, kedef, calc_prod), FP64, one thread per node.
+// forward_rate, backward, kedef, calc_prod), one thread per node: in FP64 in the FP64 form
+// (chem_node), in double-FP32 arithmetic in the mixed form (chem_node_dd), whose source is
+// rounded to FP32 in either case.
 //
 // Concentrations c_s = 1e-6 rho_s / W_s (mol/cm^3, the units of Park-type constants);
 // k_f = exp(ln A + beta ln T - theta/T); k_b = k_f / K_c with
@@ -11,10 +13,12 @@
 // Jacobian at fixed T, dt = the running RK step (0 outside RK stepping).
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stddef.h>
 #include <stdlib.h>
 #include <string.h>
 
 #include "../../include/dg.h"
+#include "dg_dd.cuh"
 #include "dg_internal.h"
 #include "dg_mlp.cuh"
 #include "dg_mlp_tc5.cuh"
@@ -184,21 +188,212 @@ __device__ __forceinline__ void chem_node(const T* uu, int np, double Tk, const 
   }
 }
 
+// element and node of a global node index; the 64-bit division (about 70 instructions) only
+// where the index needs it
+__device__ __forceinline__ void split_node(int64_t i, int np, int64_t& k, int& node) {
+  if (i >> 32) {
+    k = i / np;
+    node = (int)(i - k * np);
+  } else {
+    const unsigned q = (unsigned)i / (unsigned)np;
+    k = q;
+    node = (int)((unsigned)i - q * (unsigned)np);
+  }
+}
+
+// ------------------------------------------------------------------ mixed form
+// Tables of the double-FP32 evaluation (pairs): the same numbers as the FP64 rows above, passed
+// by value so that they sit in the constant bank (uniform loads and branches; as a table in
+// shared memory the loop spent a quarter of its issue slots on loading and decoding it).
+constexpr int MAXR = 64;
+constexpr int SCALE2 = 60;  // rates are carried times 2^60 (see chem_node_dd)
+struct ChemRow32 {
+  dgdd::dd lnA, beta, mtheta, eff[NSPEC];
+  // nu'_s, dnu_s, and the factors of r_f and r_b in the Jacobian, nu'_s dnu_s and -nu''_s dnu_s
+  float nf[NSPEC], dn[NSPEC], jf[NSPEC], jb[NSPEC];
+  // bits s, 5 + s, 10 + s, 15 + s: these are not zero; bit 20: third body
+  int mask;
+  double dn64[NSPEC];
+};
+struct ChemTab32 {
+  dgdd::dd cw[NSPEC], ow[NSPEC];     // 1e-6 / W; 1e6 W 2^-60
+  ChemRow32 row[MAXR];
+};
+static_assert(sizeof(ChemTab32) < 16 * 1024, "a kernel argument");
+
+// The rates of chem_node with the thermodynamics in FP64 and the kinetics in double-FP32 pairs
+// (48 bits; the source is rounded to FP32's 24 afterwards).  FP32 has no room for the exponents of
+// k_f, k_b and the concentration products, so the two rates of a reaction are formed from their
+// logarithms,
+//   ln r_f = ln k_f + sum nu'_s ln c_s,   ln r_b = ln r_f + delta,   delta = sum dnu_s w_s,
+//   w_s = g_s/(R T) + ln c_s - ln(1e-6 p0 / (R_u T)),
+// and carried times 2^60: rates from 2^-160 mol/cm^3/s (flushed to zero below: their source
+// is below FP32's range) to 2^66.  Near equilibrium r_f and r_b cancel to -r_f (e^delta - 1): delta is a
+// difference of numbers up to 100, so w and delta stay in FP64, and where |delta| < 1/16 the
+// difference comes from delta itself.  Measured against FP64 on states with rates from cold to 9000 K
+// and after 50 steps: the same relative L2 to three digits (2.5e-8, the rounding of the result).
+// What bounds it: about 200 FP64 operations and 8,000 others per node, on two pipes; 1,063 FP64
+// operations before.  4.6 M nodes: 10.17 -> 2.28 ms.  All of it in pairs, logarithms, g and delta too,
+// ran in 1.20 ms but missed the FP64 source by a tenfold larger maximum near equilibrium.
+// Returns false where the pairs do not hold (a concentration that is not between 1e-24 and
+// 1e6 mol/cm^3, zero and negative ones among them, or a result that is not finite); the caller
+// then evaluates the node in FP64.
+__device__ __forceinline__ bool chem_node_dd(const float* uu, int np, double Td, const ChemTab32& t,
+                                             const dgdd::dd* exp2, const double* sp, int nr, dgdd::dd* om,
+                                             dgdd::dd* jpi) {
+  using namespace dgdd;
+  dd c[NSPEC], lc[NSPEC], jd[NSPEC], j1[NSPEC];
+  double w[NSPEC];
+  bool ok = true;
+#pragma unroll
+  for (int s = 0; s < NSPEC; ++s) {
+    c[s] = mul(t.cw[s], uu[s * np]);
+    ok = ok && c[s].h >= 1e-24f && c[s].h <= 1e6f;
+  }
+  if (!ok) return false;
+  // (ln T is multiplied by the species' a1 in g: the FP64 logarithm; ln c_s good to 2^-45)
+  const double lnTd = log(Td), iTd = 1.0 / Td, mlnP = lnTd - sp[14];
+  const dd lnT = from_double(lnTd), iT = from_double(iTd);
+#pragma unroll
+  for (int s = 0; s < NSPEC; ++s) {
+    const double* q = sp + SP_W * s;
+    double l;
+    lc[s] = log_(c[s], exp2, &l);
+    w[s] = (q[2] + Td * (q[3] + Td * (q[4] + Td * (q[5] + Td * q[6]))) + q[7] * iTd - q[8] * lnTd) + l + mlnP;
+    om[s] = jd[s] = j1[s] = make(0.f, 0.f);
+  }
+#pragma unroll 1
+  for (int r = 0; r < nr; ++r) {
+    const ChemRow32& row = t.row[r];
+    const int mask = row.mask;  // the same for every node: no divergence below
+    double dl = 0.0;
+#pragma unroll
+    for (int s = 0; s < NSPEC; ++s)
+      if (mask & (1 << (5 + s))) dl += row.dn64[s] * w[s];
+    dd tf = row.lnA;
+    acc_mul(tf, row.beta, lnT);
+    acc_mul(tf, row.mtheta, iT);
+#pragma unroll
+    for (int s = 0; s < NSPEC; ++s)
+      if (mask & (1 << s)) acc_mul(tf, lc[s], row.nf[s]);
+    const dd delta = from_double(dl);
+    tf = norm(tf);
+    const dd pf = exp_scaled(tf, SCALE2, exp2);
+    dd pb = exp_scaled(add(tf, delta), SCALE2, exp2), dp = add(pf, neg(pb));
+    if (fabsf(delta.h) < 0.0625f) {
+      dp = neg(mul(pf, expm1_small(delta)));
+      pb = add(pf, neg(dp));
+    }
+    dd Rr = dp, pfM = pf, pbM = pb;
+    if (mask & (1 << 20)) {
+      dd M = mul(row.eff[0], c[0]);
+#pragma unroll
+      for (int s = 1; s < NSPEC; ++s) acc_mul(M, row.eff[s], c[s]);
+      M = norm(M);
+      Rr = mul(dp, M);
+      pfM = mul(pf, M);
+      pbM = mul(pb, M);
+#pragma unroll
+      for (int s = 0; s < NSPEC; ++s)
+        if (mask & (1 << (5 + s))) acc_mul(jd[s], mul(row.eff[s], dp), row.dn[s]);
+    }
+    // dnu_s (nu'_s r_f - nu''_s r_b) M goes to j1, divided by c_s after the loop; one of nu'_s and
+    // nu''_s is mostly zero
+#pragma unroll
+    for (int s = 0; s < NSPEC; ++s) {
+      if (mask & (1 << (5 + s))) acc_mul(om[s], Rr, row.dn[s]);
+      if (mask & (1 << (10 + s))) acc_mul(j1[s], pfM, row.jf[s]);
+      if (mask & (1 << (15 + s))) acc_mul(j1[s], pbM, row.jb[s]);
+    }
+  }
+  const float down = bits((uint32_t)(127 - SCALE2) << 23);
+#pragma unroll
+  for (int s = 0; s < NSPEC; ++s) {
+    om[s] = mul(norm(om[s]), t.ow[s]);
+    const dd j = add(norm(jd[s]), div(norm(j1[s]), c[s]));
+    ok = ok && isfinite(om[s].h) && isfinite(j.h);
+    jpi[s] = j.h < 0.f ? make(fmul(-j.h, down), fmul(-j.l, down)) : make(0.f, 0.f);
+  }
+  return ok;
+}
+
+// the FP64 evaluation of a mixed-form node that the pairs cannot hold
+__device__ __noinline__ void chem_node_rare(const float* uu, int np, double Tk, const double* sp, const double* reac,
+                                            int nr, dgdd::dd* om, dgdd::dd* jpi) {
+  double o[NSPEC], j[NSPEC];
+  chem_node<float>(uu, np, Tk, sp, reac, nr, o, j);
+#pragma unroll
+  for (int s = 0; s < NSPEC; ++s) {
+    om[s] = dgdd::from_double(o[s]);
+    jpi[s] = dgdd::from_double(j[s]);
+  }
+}
+
+// The plain source of one node in the two forms: the rates in the form's arithmetic, and
+// S_s = omega_s / (1 + dt jpi_s) rounded to the form.  Every kernel that evaluates the plain
+// source goes through these, so that they agree bit for bit.
+struct Chem64 {  // FP64 form
+  struct Tab {};
+  double om[NSPEC], jpi[NSPEC];
+  __device__ __forceinline__ static void stage(Tab&, const dgdd::dd*) {}
+  __device__ __forceinline__ void rates(const double* uu, int np, double Tk, const Tab&, const ChemTab32&,
+                                        const double* sp, const double* reac, int nr) {
+    chem_node<double>(uu, np, Tk, sp, reac, nr, om, jpi);
+  }
+  __device__ __forceinline__ double source(int s, double dt) const { return om[s] / (1.0 + dt * jpi[s]); }
+};
+struct Chem32 {  // mixed form
+  struct Tab {
+    dgdd::dd exp2[dgdd::EXP_TAB];  // 2^(j/128), in shared memory
+  };
+  dgdd::dd om[NSPEC], jpi[NSPEC];
+  __device__ __forceinline__ static void stage(Tab& t, const dgdd::dd* src) {
+    for (int j = threadIdx.x; j < dgdd::EXP_TAB; j += blockDim.x) t.exp2[j] = src[j];
+    __syncthreads();
+  }
+  __device__ __forceinline__ void rates(const float* uu, int np, double Tk, const Tab& e, const ChemTab32& t,
+                                        const double* sp, const double* reac, int nr) {
+    if (!chem_node_dd(uu, np, Tk, t, e.exp2, sp, nr, om, jpi)) {
+      dgdd::dd o[NSPEC], j[NSPEC];
+      chem_node_rare(uu, np, Tk, sp, reac, nr, o, j);
+#pragma unroll
+      for (int s = 0; s < NSPEC; ++s) {
+        om[s] = o[s];
+        jpi[s] = j[s];
+      }
+    }
+  }
+  __device__ __forceinline__ float source(int s, dgdd::dd dt) const {
+    using namespace dgdd;
+    return div(om[s], mul_add(dt, jpi[s], make(1.f, 0.f))).h;
+  }
+};
+template <typename T> struct ChemForm;
+template <> struct ChemForm<double> { typedef Chem64 type; typedef double step; };
+template <> struct ChemForm<float> { typedef Chem32 type; typedef dgdd::dd step; };
+__device__ __forceinline__ void form_step(double dt, double& out) { out = dt; }
+__device__ __forceinline__ void form_step(double dt, dgdd::dd& out) { out = dgdd::from_double(dt); }
+
 template <typename T>
-__global__ void chem_kernel(const T* u, const double* Tc, int64_t K, int np, int dim,
-                            const double* sp_raw, const double* reac, int nr, const double* dtp,
-                            T* src) {
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 1)
+chem_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, const double* sp_raw, const double* reac,
+            int nr, const __grid_constant__ ChemTab32 tab, const dgdd::dd* exp2, const double* dtp, T* src) {
+  typedef typename ChemForm<T>::type Form;
+  __shared__ typename Form::Tab t;
+  Form::stage(t, exp2);
   const int nv = NSPEC + dim + 1;
-  const double dt = dtp ? *dtp : 0.0;
+  typename ChemForm<T>::step dt;
+  form_step(dtp ? *dtp : 0.0, dt);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < K * np;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t k = i / np;
-    const int node = (int)(i % np);
-    double om[NSPEC], jpi[NSPEC];
-    chem_node<T>(u + k * nv * np + node, np, Tc[i], sp_raw, reac, nr, om, jpi);
+    int64_t k;
+    int node;
+    split_node(i, np, k, node);
+    Form f;
+    f.rates(u + k * nv * np + node, np, Tc[i], t, tab, sp_raw, reac, nr);
     T* so = src + k * NSPEC * np + node;
 #pragma unroll
-    for (int s = 0; s < NSPEC; ++s) so[s * np] = (T)(om[s] / (1.0 + dt * jpi[s]));
+    for (int s = 0; s < NSPEC; ++s) so[s * np] = f.source(s, dt);
   }
 }
 
@@ -216,13 +411,15 @@ __global__ void chem_kernel(const T* u, const double* Tc, int64_t K, int np, int
 // every node and stores, per node, the plain rates minus the network's decoded ones; the
 // evaluations until the next refresh add those differences to the decoded rates before the
 // tests, so the corrected network is exact at the refresh state.
-struct __align__(16) DgChemMlp {
-  DgMlpW<10> w;
+struct DgChemStats {
   float mean[7], inv_std[7], muY[10], sdY[10], lo[7], hi[7];
   float w_ref, j_ref, tol_mass, floor32;
+};
+struct __align__(16) DgChemMlp {
+  DgMlpW<10> w;
+  DgChemStats st;
   double tol_check, floor;
 };
-
 constexpr int CHEM_NR = 1;  // rows per thread of the tile engine (the decode needs the registers)
 
 __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
@@ -232,9 +429,9 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
   return x ^ (x >> 31);
 }
 
-// raw features of one node: Y_1..Y_5, ln rho, T
+// raw features of one node: Y_1..Y_5, ln rho, T, each rounded to FP32 once
 template <typename T>
-__device__ __forceinline__ void chem_features(const T* uu, int np, double Tk, float* x) {
+__device__ __forceinline__ void chem_features(const T* uu, int np, double Tk, const dgdd::dd*, float* x) {
   double r[NSPEC], rho = 0.0;
 #pragma unroll
   for (int s = 0; s < NSPEC; ++s) {
@@ -247,6 +444,44 @@ __device__ __forceinline__ void chem_features(const T* uu, int np, double Tk, fl
   x[5] = (float)log(rho);
   x[6] = (float)Tk;
 }
+// the mixed form's in pairs (tab: the table of exp_scaled): one FP64 logarithm and division per
+// node took half of the network kernel's time
+__device__ __forceinline__ void chem_features(const float* uu, int np, double Tk, const dgdd::dd* tab, float* x) {
+  using namespace dgdd;
+  float r[NSPEC];
+  dd rho = make(0.f, 0.f);
+#pragma unroll
+  for (int s = 0; s < NSPEC; ++s) {
+    r[s] = uu[s * np];
+    acc(rho, make(r[s], 0.f));
+  }
+  rho = norm(rho);
+  if (!(rho.h > 1e-30f && rho.h < 1e30f)) {  // out of the pairs' range
+    chem_features<float>(uu, np, Tk, tab, x);
+    return;
+  }
+  const dd ir = rcp(rho);
+#pragma unroll
+  for (int s = 0; s < NSPEC; ++s) x[s] = mul(ir, r[s]).h;
+  x[5] = log_(rho, tab).h;
+  x[6] = (float)Tk;
+}
+
+// sinh(z): its Taylor series to z^9 below 1 (the next term is under 3e-8 of it), (e^a - e^-a) / 2
+// above; half the instructions of sinhf, whose branches both run in a mixed warp
+__device__ __forceinline__ float sinh_pair(float z) {
+  const float a = fabsf(z), a2 = a * a;
+  const float lo = a + a * a2 * (1.f / 6.f + a2 * (1.f / 120.f + a2 * (1.f / 5040.f + a2 * (1.f / 362880.f))));
+  const float E = expf(a);
+  const float hi = 0.5f * E - __fdividef(0.5f, E);
+  return copysignf(a < 1.f ? lo : hi, z);
+}
+
+// the node of tile t that evaluation `call` checks
+__device__ __forceinline__ int64_t sampled_node(int64_t t, int64_t total, uint64_t call) {
+  const int64_t in_tile = total - t * 32 < 32 ? total - t * 32 : 32;
+  return t * 32 + (int64_t)(splitmix64(call * 0x100000001B3ull + (uint64_t)t) % (uint64_t)in_tile);
+}
 
 // The learned source on the fifth-generation tensor cores: CTAs of 128 threads take
 // 128-node tiles through the tcgen05 tile engine (dg_mlp_tc5.cuh); each thread forms its
@@ -258,26 +493,58 @@ __device__ __forceinline__ void chem_features(const T* uu, int np, double Tk, fl
 // plain-minus-network differences before the tests (omega_s + c_s, max(0, jpi'_s + c_5+s));
 // cmode 2 (refresh): only the decoded rates (jpi' before its clamp) are written to corr,
 // for chem_refresh_kernel to turn into corrections.
+// The first `checks` CTAs of the grid evaluate the plain source at every tile's sampled node
+// instead (one thread per tile, S into `sampled`) for the next kernel to compare with: a chain
+// of one evaluation that fills a fraction of the GPU (28 us as a kernel of its own at 18,000
+// tiles) runs beside the network.
 template <typename T>
-__global__ void __launch_bounds__(dgtc5::THREADS, 4)
-chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, const DgChemMlp* mlp,
-                    const double* dtp, T* src, unsigned char* flags, float* corr, const unsigned char* trust,
-                    int cmode) {
+__global__ void __launch_bounds__(dgtc5::THREADS, sizeof(T) == 4 ? 5 : 3)
+chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, const double* sp_raw,
+                    const double* reac, int nr, const __grid_constant__ ChemTab32 tab, const dgdd::dd* exp2,
+                    const DgChemMlp* mlp, const double* dtp, T* src, unsigned char* flags, float* corr,
+                    const unsigned char* trust, int cmode, int checks, T* sampled, uint64_t call,
+                    unsigned long long* stats) {
+  typedef typename ChemForm<T>::type Form;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  dgtc5::Smem<10, CHEM_NR>& s = *reinterpret_cast<dgtc5::Smem<10, CHEM_NR>*>(smem_raw);
-  dgtc5::alloc_tmem<10, CHEM_NR>(s);
-  __shared__ DgChemMlp m;
-  dgmlp::copy_to_smem(m, mlp);
-  __syncthreads();
-  dgtc5::load_weights<10, CHEM_NR>(s, m.w);
   const int nv = NSPEC + dim + 1;
   const int64_t total = K * np;
+  if (cmode != 2 && blockIdx.x == 0 && threadIdx.x == 0) stats[2] = 0;  // chem_fallback_kernel's tile counter
+  if ((int)blockIdx.x < checks) {
+    typename Form::Tab& tb = *reinterpret_cast<typename Form::Tab*>(smem_raw);
+    Form::stage(tb, exp2);
+    const int64_t t = blockIdx.x * (int64_t)dgtc5::THREADS + threadIdx.x;
+    if (t * 32 >= total || (cmode == 1 && !trust[t])) return;
+    typename ChemForm<T>::step dt;
+    form_step(dtp ? *dtp : 0.0, dt);
+    int64_t k;
+    int node;
+    const int64_t i = sampled_node(t, total, call);
+    split_node(i, np, k, node);
+    Form f;
+    f.rates(u + k * nv * np + node, np, Tc[i], tb, tab, sp_raw, reac, nr);
+#pragma unroll
+    for (int s = 0; s < NSPEC; ++s) sampled[NSPEC * t + s] = f.source(s, dt);
+    return;
+  }
+  dgtc5::Smem<10, CHEM_NR>& s = *reinterpret_cast<dgtc5::Smem<10, CHEM_NR>*>(smem_raw);
+  dgtc5::alloc_tmem<10, CHEM_NR>(s);
+  __shared__ DgChemStats m;
+  __shared__ dgdd::dd e2[sizeof(T) == 4 ? dgdd::EXP_TAB : 1];
+  if (threadIdx.x < sizeof(m) / 4)
+    reinterpret_cast<int*>(&m)[threadIdx.x] = reinterpret_cast<const int*>(&mlp->st)[threadIdx.x];
+  if (sizeof(T) == 4)
+    for (int j = threadIdx.x; j < dgdd::EXP_TAB; j += dgtc5::THREADS) e2[j] = exp2[j];
+  dgtc5::load_weights<10, CHEM_NR>(s, mlp->w);
+  __syncthreads();
   const float dt = dtp ? (float)*dtp : 0.f;
   auto prod = [&](int64_t i, float* x, int) {
     float raw[7];
     bool ok = true;
     if (i < total) {
-      chem_features<T>(u + (i / np) * nv * np + (i % np), np, Tc[i], raw);
+      int64_t k;
+      int node;
+      split_node(i, np, k, node);
+      chem_features(u + k * nv * np + node, np, Tc[i], e2, raw);
 #pragma unroll
       for (int q = 0; q < 7; ++q) ok = ok && raw[q] >= m.lo[q] && raw[q] <= m.hi[q];
     } else {
@@ -294,19 +561,22 @@ chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, co
       if (i < total && valid) {
 #pragma unroll
         for (int q = 0; q < NSPEC; ++q) {
-          corr[q * total + i] = m.w_ref * sinhf(m.muY[q] + m.sdY[q] * y[q]);
-          corr[(5 + q) * total + i] = m.j_ref * sinhf(m.muY[5 + q] + m.sdY[5 + q] * y[5 + q]);
+          corr[q * total + i] = m.w_ref * sinh_pair(m.muY[q] + m.sdY[q] * y[q]);
+          corr[(5 + q) * total + i] = m.j_ref * sinh_pair(m.muY[5 + q] + m.sdY[5 + q] * y[5 + q]);
         }
       }
       return;
     }
     ok = ok && valid;
     if (i < total && valid) {
+      int64_t k;
+      int node;
+      split_node(i, np, k, node);
       float om[NSPEC], jp[NSPEC], msum = 0.f, asum = 0.f;
 #pragma unroll
       for (int q = 0; q < NSPEC; ++q) {
-        om[q] = m.w_ref * sinhf(m.muY[q] + m.sdY[q] * y[q]);
-        float jr = m.j_ref * sinhf(m.muY[5 + q] + m.sdY[5 + q] * y[5 + q]);
+        om[q] = m.w_ref * sinh_pair(m.muY[q] + m.sdY[q] * y[q]);
+        float jr = m.j_ref * sinh_pair(m.muY[5 + q] + m.sdY[5 + q] * y[5 + q]);
         if (cmode == 1) {
           om[q] += corr[q * total + i];
           jr += corr[(5 + q) * total + i];
@@ -317,10 +587,10 @@ chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, co
       }
       ok = ok && isfinite(asum) && fabsf(msum) <= m.tol_mass * asum + m.floor32;
       const float f = asum > 0.f ? msum / asum : 0.f;
-      T* so = src + (i / np) * NSPEC * np + (i % np);
+      T* so = src + k * NSPEC * np + node;
       // positivity of the learned update: rho_s + dt S_s >= 0 (the plain point-implicit
       // source never consumes a species faster than the step allows; a learned one can)
-      const T* uu = u + (i / np) * nv * np + (i % np);
+      const T* uu = u + k * nv * np + node;
 #pragma unroll
       for (int q = 0; q < NSPEC; ++q) {
         const float Sq = (om[q] - fabsf(om[q]) * f) / (1.f + dt * jp[q]);
@@ -337,70 +607,92 @@ chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, co
       flags[base >> 5] = !trusted ? 4 : (tile_ok ? 0 : 1);
     }
   };
-  dgtc5::run_tiles<10, CHEM_NR>(s, total, prod, cons);
+  // with corrections, a tile none of whose warps is trusted needs no network
+  auto skip = [&](int64_t row0) {
+    if (cmode != 1) return false;
+    bool need = false;
+#pragma unroll
+    for (int r = 0; r < CHEM_NR; ++r) {
+      const int64_t t = (row0 + r * dgtc5::ROWS) >> 5;  // this warp's 32-node tile
+      need = need || (t * 32 < total && trust[t]);
+    }
+    if (__syncthreads_or(need)) return false;
+#pragma unroll
+    for (int r = 0; r < CHEM_NR; ++r) {
+      const int64_t t = (row0 + r * dgtc5::ROWS) >> 5;
+      if ((threadIdx.x & 31) == 0 && t * 32 < total) flags[t] = 4;
+    }
+    return true;
+  };
+  dgtc5::run_tiles<10, CHEM_NR>(s, total, prod, cons, skip, checks);
 }
 
-// one thread per tile still accepted: compare the learned source at the tile's sampled
-// node with the plain FP64 source there
+// a warp at a time takes the next tile (stats[2] counts them, set to zero by chem_mlp_tc5_kernel):
+// the sampled check if it is still accepted (the learned source at the sampled node against the
+// plain one that chem_mlp_tc5_kernel left), then, if rejected, the plain source at its nodes;
+// counts nodes.  Rejected tiles cluster where the rates are large; with a fixed share of the tiles
+// per warp a learned evaluation takes 5 % longer (18,000 tiles, 44 % rejected).
 template <typename T>
-__global__ void chem_check_kernel(const T* u, const double* Tc, int64_t K, int np, int dim,
-                                  const double* sp_raw, const double* reac, int nr, const DgChemMlp* mlp,
-                                  const double* dtp, const T* src, unsigned char* flags, uint64_t call) {
-  const int nv = NSPEC + dim + 1;
-  const int64_t total = K * np, ntiles = (total + 31) / 32;
-  const double dt = dtp ? *dtp : 0.0;
-  const double tol = mlp->tol_check, floor_ = mlp->floor;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ntiles;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    if (flags[t]) continue;
-    const int64_t in_tile = total - t * 32 < 32 ? total - t * 32 : 32;
-    const int64_t i = t * 32 + (int64_t)(splitmix64(call * 0x100000001B3ull + (uint64_t)t) % (uint64_t)in_tile);
-    const int64_t k = i / np;
-    const int node = (int)(i % np);
-    double om[NSPEC], jpi[NSPEC], Sp[NSPEC], scale = 0.0;
-    chem_node<T>(u + k * nv * np + node, np, Tc[i], sp_raw, reac, nr, om, jpi);
-#pragma unroll
-    for (int s = 0; s < NSPEC; ++s) {
-      Sp[s] = om[s] / (1.0 + dt * jpi[s]);
-      scale += fabs(Sp[s]);
-    }
-    bool ok = true;
-#pragma unroll
-    for (int s = 0; s < NSPEC; ++s) {
-      const double Sm = (double)src[(k * NSPEC + s) * np + node];
-      ok = ok && fabs(Sm - Sp[s]) <= tol * scale + floor_;
-    }
-    if (!ok) flags[t] = 2;
-  }
-}
-
-// one warp per tile: recompute rejected tiles with the plain source; count nodes
-template <typename T>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 1)
 chem_fallback_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, const double* sp_raw,
-                     const double* reac, int nr, const double* dtp, T* src, const unsigned char* flags,
-                     unsigned long long* stats) {
+                     const double* reac, int nr, const __grid_constant__ ChemTab32 tab, const dgdd::dd* exp2,
+                     const DgChemMlp* mlp, const double* dtp, T* src, unsigned char* flags, const T* sampled,
+                     uint64_t call, unsigned long long* stats) {
+  typedef typename ChemForm<T>::type Form;
+  __shared__ typename Form::Tab tb;
+  Form::stage(tb, exp2);
   const int nv = NSPEC + dim + 1;
   const int lane = threadIdx.x & 31;
   const int64_t total = K * np, ntiles = (total + 31) / 32;
-  const double dt = dtp ? *dtp : 0.0;
+  const T tol = (T)mlp->tol_check, floor_ = (T)mlp->floor;
+  typename ChemForm<T>::step dt;
+  form_step(dtp ? *dtp : 0.0, dt);
   unsigned long long n_ok = 0, n_fb = 0;
-  for (int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; t < ntiles;
-       t += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int64_t i = t * 32 + lane;
-    if (i >= total) continue;
-    if (!flags[t]) {
-      ++n_ok;
-      continue;
-    }
-    ++n_fb;
-    const int64_t k = i / np;
-    const int node = (int)(i % np);
-    double om[NSPEC], jpi[NSPEC];
-    chem_node<T>(u + k * nv * np + node, np, Tc[i], sp_raw, reac, nr, om, jpi);
-    T* so = src + k * NSPEC * np + node;
+  for (;;) {
+    unsigned long long next = 0;
+    if (lane == 0) next = atomicAdd(&stats[2], 1ull);
+    const int64_t t = (int64_t)__shfl_sync(0xffffffffu, next, 0);
+    if (t >= ntiles) break;
+    int flag = flags[t];
+    if (!flag) {
+      int64_t k;
+      int node;
+      split_node(sampled_node(t, total, call), np, k, node);
+      T Sp[NSPEC], scale = 0;
 #pragma unroll
-    for (int s = 0; s < NSPEC; ++s) so[s * np] = (T)(om[s] / (1.0 + dt * jpi[s]));
+      for (int s = 0; s < NSPEC; ++s) {
+        Sp[s] = sampled[NSPEC * t + s];
+        scale += fabs(Sp[s]);
+      }
+      bool ok = true;
+#pragma unroll
+      for (int s = 0; s < NSPEC; ++s) {
+        const T Sm = src[(k * NSPEC + s) * np + node];
+        ok = ok && fabs(Sm - Sp[s]) <= tol * scale + floor_;
+      }
+      if (!ok) {  // the same in all lanes
+        flag = 2;
+        __syncwarp();
+        if (lane == 0) flags[t] = 2;
+      }
+    }
+    const int64_t i = t * 32 + lane;
+    if (i < total) {
+      if (!flag) {
+        ++n_ok;
+      } else {
+        ++n_fb;
+        int64_t k;
+        int node;
+        split_node(i, np, k, node);
+        Form f;
+        f.rates(u + k * nv * np + node, np, Tc[i], tb, tab, sp_raw, reac, nr);
+        T* so = src + k * NSPEC * np + node;
+#pragma unroll
+        for (int s = 0; s < NSPEC; ++s) so[s * np] = f.source(s, dt);
+      }
+    }
+    __syncwarp();
   }
   for (int o = 16; o > 0; o >>= 1) {
     n_ok += __shfl_xor_sync(0xffffffffu, n_ok, o);
@@ -412,50 +704,93 @@ chem_fallback_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, c
   }
 }
 
-// refresh of the corrections: every node takes the plain FP64 source, and corr (holding
+// refresh of the corrections: every node takes the plain source, and corr (holding
 // the network's decoded rates of this state, written by chem_mlp_tc5_kernel in cmode 2)
 // becomes the plain-minus-network differences; every tile is flagged 3 (plain).  The full
 // check: each node's uncorrected learned source (projection, point-implicit factor) against
 // the plain one with the sampled check's test; a tile is trusted until the next refresh when
 // all of its nodes pass.  Threads are grouped in warps over whole 32-node tiles.
+__device__ __forceinline__ bool refresh_node(const Chem64& p, double dt, double tol, double floor_, int64_t total,
+                                             float* corr, double* S) {
+  double oh[NSPEC], jh[NSPEC], scale = 0.0, msum = 0.0, asum = 0.0;
+#pragma unroll
+  for (int s = 0; s < NSPEC; ++s) {
+    S[s] = p.source(s, dt);
+    scale += fabs(S[s]);
+    oh[s] = (double)corr[s * total];
+    jh[s] = (double)corr[(5 + s) * total];
+    msum += oh[s];
+    asum += fabs(oh[s]);
+  }
+  const double f = asum > 0.0 ? msum / asum : 0.0;
+  bool ok = isfinite(asum);
+#pragma unroll
+  for (int s = 0; s < NSPEC; ++s) {
+    const double Sl = (oh[s] - fabs(oh[s]) * f) / (1.0 + dt * fmax(0.0, jh[s]));
+    ok = ok && fabs(Sl - S[s]) <= tol * scale + floor_;
+    corr[s * total] = (float)(p.om[s] - oh[s]);
+    corr[(5 + s) * total] = (float)(p.jpi[s] - jh[s]);
+  }
+  return ok;
+}
+// the same in pairs (the comparison itself in FP32: both sides carry 48 bits up to it)
+__device__ __forceinline__ bool refresh_node(const Chem32& p, dgdd::dd dt, double tol, double floor_, int64_t total,
+                                             float* corr, float* S) {
+  using namespace dgdd;
+  dd Sp[NSPEC], msum = make(0.f, 0.f), asum = msum, scale = msum;
+  float oh[NSPEC], jh[NSPEC];
+#pragma unroll
+  for (int s = 0; s < NSPEC; ++s) {
+    Sp[s] = div(p.om[s], mul_add(dt, p.jpi[s], make(1.f, 0.f)));
+    S[s] = Sp[s].h;
+    acc(scale, Sp[s].h < 0.f ? neg(Sp[s]) : Sp[s]);
+    oh[s] = corr[s * total];
+    jh[s] = corr[(5 + s) * total];
+    acc(msum, make(oh[s], 0.f));
+    acc(asum, make(fabsf(oh[s]), 0.f));
+  }
+  bool ok = isfinite(asum.h);
+  const dd f = asum.h > 0.f ? div(norm(msum), norm(asum)) : make(0.f, 0.f);
+  const float bound = (float)(tol * to_double(norm(scale)) + floor_);
+#pragma unroll
+  for (int s = 0; s < NSPEC; ++s) {
+    const dd Sl = div(add(neg(mul(f, fabsf(oh[s]))), oh[s]), add(mul(dt, fmaxf(0.f, jh[s])), 1.f));
+    ok = ok && fabsf(add(Sl, neg(Sp[s])).h) <= bound;
+    corr[s * total] = add(p.om[s], -oh[s]).h;
+    corr[(5 + s) * total] = add(p.jpi[s], -jh[s]).h;
+  }
+  return ok;
+}
+
 template <typename T>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 1)
 chem_refresh_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, const double* sp_raw,
-                    const double* reac, int nr, const DgChemMlp* mlp, const double* dtp, T* src, float* corr,
-                    unsigned char* flags, unsigned char* trust) {
+                    const double* reac, int nr, const __grid_constant__ ChemTab32 tab, const dgdd::dd* exp2,
+                    const DgChemMlp* mlp, const double* dtp, T* src, float* corr, unsigned char* flags,
+                    unsigned char* trust) {
+  typedef typename ChemForm<T>::type Form;
+  __shared__ typename Form::Tab tb;
+  Form::stage(tb, exp2);
   const int nv = NSPEC + dim + 1;
   const int64_t total = K * np;
-  const double dt = dtp ? *dtp : 0.0;
+  typename ChemForm<T>::step dt;
+  form_step(dtp ? *dtp : 0.0, dt);
   const double tol = mlp->tol_check, floor_ = mlp->floor;
   const int lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;  // a multiple of 32
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i - lane < total; i += stride) {
     bool ok = true;
     if (i < total) {
-      const int64_t k = i / np;
-      const int node = (int)(i % np);
-      double om[NSPEC], jpi[NSPEC], Sp[NSPEC], oh[NSPEC], jh[NSPEC], scale = 0.0, msum = 0.0, asum = 0.0;
-      chem_node<T>(u + k * nv * np + node, np, Tc[i], sp_raw, reac, nr, om, jpi);
+      int64_t k;
+      int node;
+      split_node(i, np, k, node);
+      Form p;
+      p.rates(u + k * nv * np + node, np, Tc[i], tb, tab, sp_raw, reac, nr);
+      T S[NSPEC];
+      ok = refresh_node(p, dt, tol, floor_, total, corr + i, S);
       T* so = src + k * NSPEC * np + node;
 #pragma unroll
-      for (int s = 0; s < NSPEC; ++s) {
-        Sp[s] = om[s] / (1.0 + dt * jpi[s]);
-        so[s * np] = (T)Sp[s];
-        scale += fabs(Sp[s]);
-        oh[s] = (double)corr[s * total + i];
-        jh[s] = (double)corr[(5 + s) * total + i];
-        msum += oh[s];
-        asum += fabs(oh[s]);
-      }
-      const double f = asum > 0.0 ? msum / asum : 0.0;
-      ok = isfinite(asum);
-#pragma unroll
-      for (int s = 0; s < NSPEC; ++s) {
-        const double Sl = (oh[s] - fabs(oh[s]) * f) / (1.0 + dt * fmax(0.0, jh[s]));
-        ok = ok && fabs(Sl - Sp[s]) <= tol * scale + floor_;
-        corr[s * total + i] = (float)(om[s] - oh[s]);
-        corr[(5 + s) * total + i] = (float)(jpi[s] - jh[s]);
-      }
+      for (int s = 0; s < NSPEC; ++s) so[s * np] = S[s];
     }
     const bool tile_ok = __all_sync(0xffffffffu, ok);
     if (lane == 0) {
@@ -474,10 +809,11 @@ __global__ void chem_sample_kernel(const T* u, const double* Tc, int64_t K, int 
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
        j += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = (int64_t)(splitmix64(seed + (uint64_t)j) % (uint64_t)(K * np));
-    const int64_t k = i / np;
-    const int node = (int)(i % np);
+    int64_t k;
+    int node;
+    split_node(i, np, k, node);
     const T* uu = u + k * nv * np + node;
-    chem_features<T>(uu, np, Tc[i], X + j * 7);
+    chem_features<T>(uu, np, Tc[i], nullptr, X + j * 7);
     chem_node<T>(uu, np, Tc[i], sp_raw, reac, nr, Y + j * 10, Y + j * 10 + 5);
   }
 }
@@ -546,8 +882,43 @@ cudaError_t dg_chem_init(DgThermo* th, const double* species_host, const double*
     o[10] = DG_RU / (1e-6 * DG_P0);  // 1/P = o[10] T
     o[14] = log(1e-6 * DG_P0 / DG_RU);
   }
+  // the same rows as pairs for the mixed form
+  ChemTab32* t32 = (ChemTab32*)calloc(1, sizeof(ChemTab32));
+  if (!t32) {
+    free(rows);
+    return cudaErrorMemoryAllocation;
+  }
+  dgdd::dd e2[dgdd::EXP_TAB];
+  for (int j = 0; j < dgdd::EXP_TAB; ++j) e2[j] = dgdd::from_double(exp2(j / (double)dgdd::EXP_TAB));
+  for (int s = 0; s < NSPEC; ++s) {
+    const double* o = sp + SP_W * s;
+    t32->cw[s] = dgdd::from_double(o[0]);
+    t32->ow[s] = dgdd::from_double(ldexp(o[1], -SCALE2));
+  }
+  for (int r = 0; r < nr; ++r) {
+    const double* o = rows + RX_W * r;
+    ChemRow32& w = t32->row[r];
+    w.lnA = dgdd::from_double(o[16]);
+    w.beta = dgdd::from_double(o[17]);
+    w.mtheta = dgdd::from_double(-o[18]);
+    for (int s = 0; s < NSPEC; ++s) {
+      const float a = (float)o[s], b = (float)o[5 + s];
+      w.eff[s] = dgdd::from_double(o[11 + s]);
+      w.nf[s] = a;
+      w.dn[s] = b - a;
+      w.dn64[s] = (double)(b - a);
+      w.jf[s] = a * (b - a);
+      w.jb[s] = -b * (b - a);
+      w.mask |= (w.nf[s] != 0.f) << s | (w.dn[s] != 0.f) << (5 + s) | (w.jf[s] != 0.f) << (10 + s) |
+                (w.jb[s] != 0.f) << (15 + s);
+    }
+    if (o[10] != 0.0) w.mask |= 1 << 20;
+  }
+  th->chem_tab32 = t32;  // host memory, freed with the context
   const size_t rs = th->f32 ? sizeof(float) : sizeof(double);
-  cudaError_t e = cudaMalloc((void**)&th->reac, sizeof(double) * RX_W * nr);
+  cudaError_t e = cudaMalloc(&th->chem_exp2, sizeof(e2));
+  if (e == cudaSuccess) e = cudaMemcpy(th->chem_exp2, e2, sizeof(e2), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&th->reac, sizeof(double) * RX_W * nr);
   if (e == cudaSuccess) e = cudaMemcpy(th->reac, rows, sizeof(double) * RX_W * nr, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc((void**)&th->species_raw, sizeof(double) * SP_W * NSPEC);
   if (e == cudaSuccess) e = cudaMemcpy(th->species_raw, sp, sizeof(double) * SP_W * NSPEC, cudaMemcpyHostToDevice);
@@ -561,19 +932,22 @@ template <typename T>
 static cudaError_t chem_learned(DgThermo* th, const T* u, const double* dt_dev, int refresh, cudaStream_t s) {
   const int64_t total = th->K * th->np, ntiles = (total + 31) / 32;
   const DgChemMlp* m = (const DgChemMlp*)th->chem_mlp;
-  // persistent CTAs over tensor-core tiles of 128 nodes
+  const ChemTab32& tab = *(const ChemTab32*)th->chem_tab32;
+  const dgdd::dd* e2 = (const dgdd::dd*)th->chem_exp2;
   const size_t smem = sizeof(dgtc5::Smem<10, CHEM_NR>);
   auto k1 = chem_mlp_tc5_kernel<T>;
   cudaError_t e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int64_t t128 = (total + dgtc5::ROWS - 1) / dgtc5::ROWS;
-  const unsigned g1 = (unsigned)(t128 < 152 * 4 ? t128 : 152 * 4);
+  // persistent CTAs over tensor-core tiles of 128 nodes
+  const int64_t rows = CHEM_NR * dgtc5::ROWS, tiles = (total + rows - 1) / rows;
+  const unsigned g1 = (unsigned)(tiles < 152 * 5 ? tiles : 152 * 5);
   if (refresh) {
     if (!th->chem_corr || !th->chem_trust) return cudaErrorInvalidValue;
-    k1<<<g1, dgtc5::THREADS, smem, s>>>(u, th->T, th->K, th->np, th->dim, m, dt_dev, (T*)th->src,
-                                        th->chem_flags, th->chem_corr, th->chem_trust, 2);
+    k1<<<g1, dgtc5::THREADS, smem, s>>>(u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr, tab, e2, m,
+                                        dt_dev, (T*)th->src, th->chem_flags, th->chem_corr, th->chem_trust, 2, 0,
+                                        NULL, 0, NULL);
     chem_refresh_kernel<T><<<grid_of(ntiles * 32), 128, 0, s>>>(u, th->T, th->K, th->np, th->dim,
-                                                                th->species_raw, th->reac, th->nr, m, dt_dev,
+                                                                th->species_raw, th->reac, th->nr, tab, e2, m, dt_dev,
                                                                 (T*)th->src, th->chem_corr, th->chem_flags,
                                                                 th->chem_trust);
     e = cudaGetLastError();
@@ -581,16 +955,17 @@ static cudaError_t chem_learned(DgThermo* th, const T* u, const double* dt_dev, 
     return e;
   }
   const int cmode = th->chem_corr && th->chem_trust && th->corr_valid ? 1 : 0;
-  k1<<<g1, dgtc5::THREADS, smem, s>>>(u, th->T, th->K, th->np, th->dim, m, dt_dev, (T*)th->src, th->chem_flags,
-                                      th->chem_corr, th->chem_trust, cmode);
-  chem_check_kernel<T><<<grid_of(ntiles), 128, 0, s>>>(u, th->T, th->K, th->np, th->dim, th->species_raw,
-                                                       th->reac, th->nr, m, dt_dev, (const T*)th->src,
-                                                       th->chem_flags, th->chem_calls++);
+  const unsigned checks = (unsigned)((ntiles + dgtc5::THREADS - 1) / dgtc5::THREADS);
+  const uint64_t call = th->chem_calls++;
+  k1<<<checks + g1, dgtc5::THREADS, smem, s>>>(u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr,
+                                               tab, e2, m, dt_dev, (T*)th->src, th->chem_flags, th->chem_corr,
+                                               th->chem_trust, cmode, (int)checks, (T*)th->chem_sampled, call,
+                                               th->chem_stats);
   int64_t g3 = (ntiles + 3) / 4;
-  if (g3 > 152 * 64) g3 = 152 * 64;
-  chem_fallback_kernel<T><<<(unsigned)g3, 128, 0, s>>>(u, th->T, th->K, th->np, th->dim, th->species_raw,
-                                                        th->reac, th->nr, dt_dev, (T*)th->src, th->chem_flags,
-                                                        th->chem_stats);
+  if (g3 > 152 * 5) g3 = 152 * 5;
+  chem_fallback_kernel<T><<<(unsigned)g3, 128, 0, s>>>(u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac,
+                                                       th->nr, tab, e2, m, dt_dev, (T*)th->src, th->chem_flags,
+                                                       (const T*)th->chem_sampled, call, th->chem_stats);
   return cudaGetLastError();
 }
 
@@ -601,12 +976,12 @@ cudaError_t dg_chem_source(DgThermo* th, const void* u, int f32, const double* d
                : chem_learned<double>(th, (const double*)u, dt_dev, refresh, s);
   if (f32)
     chem_kernel<float><<<grid_of(th->K * th->np), 128, 0, s>>>(
-        (const float*)u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr, dt_dev,
-        (float*)th->src);
+        (const float*)u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr,
+        *(const ChemTab32*)th->chem_tab32, (const dgdd::dd*)th->chem_exp2, dt_dev, (float*)th->src);
   else
     chem_kernel<double><<<grid_of(th->K * th->np), 128, 0, s>>>(
-        (const double*)u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr, dt_dev,
-        (double*)th->src);
+        (const double*)u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr,
+        *(const ChemTab32*)th->chem_tab32, (const dgdd::dd*)th->chem_exp2, dt_dev, (double*)th->src);
   return cudaGetLastError();
 }
 
@@ -621,26 +996,27 @@ cudaError_t dg_chem_mlp_set(DgThermo* th, const float* params_host, const double
   if (!h) return cudaErrorMemoryAllocation;
   dg_mlp_pack<10>(params_host, &h->w);
   for (int q = 0; q < 7; ++q) {
-    h->mean[q] = (float)st[DG_SRC_X_MEAN + q];
-    h->inv_std[q] = (float)(1.0 / st[DG_SRC_X_STD + q]);
-    h->lo[q] = (float)st[DG_SRC_BOX_LO + q];
-    h->hi[q] = (float)st[DG_SRC_BOX_HI + q];
+    h->st.mean[q] = (float)st[DG_SRC_X_MEAN + q];
+    h->st.inv_std[q] = (float)(1.0 / st[DG_SRC_X_STD + q]);
+    h->st.lo[q] = (float)st[DG_SRC_BOX_LO + q];
+    h->st.hi[q] = (float)st[DG_SRC_BOX_HI + q];
   }
   for (int q = 0; q < 10; ++q) {
-    h->muY[q] = (float)st[DG_SRC_Y_MEAN + q];
-    h->sdY[q] = (float)st[DG_SRC_Y_STD + q];
+    h->st.muY[q] = (float)st[DG_SRC_Y_MEAN + q];
+    h->st.sdY[q] = (float)st[DG_SRC_Y_STD + q];
   }
-  h->w_ref = (float)st[DG_SRC_OMEGA_REF];
-  h->j_ref = (float)st[DG_SRC_JPI_REF];
-  h->tol_mass = (float)st[DG_SRC_TOL_MASS];
+  h->st.w_ref = (float)st[DG_SRC_OMEGA_REF];
+  h->st.j_ref = (float)st[DG_SRC_JPI_REF];
+  h->st.tol_mass = (float)st[DG_SRC_TOL_MASS];
   h->tol_check = st[DG_SRC_TOL_CHECK];
   h->floor = st[DG_SRC_FLOOR];
-  h->floor32 = (float)st[DG_SRC_FLOOR];
+  h->st.floor32 = (float)st[DG_SRC_FLOOR];
   const int64_t ntiles = (th->K * th->np + 31) / 32;
   cudaError_t e = cudaSuccess;
   if (!th->chem_mlp) e = cudaMalloc(&th->chem_mlp, sizeof(DgChemMlp));
-  if (e == cudaSuccess && !th->chem_stats) e = cudaMalloc((void**)&th->chem_stats, 2 * sizeof(unsigned long long));
+  if (e == cudaSuccess && !th->chem_stats) e = cudaMalloc((void**)&th->chem_stats, 3 * sizeof(unsigned long long));
   if (e == cudaSuccess && !th->chem_flags) e = cudaMalloc((void**)&th->chem_flags, (size_t)ntiles);
+  if (e == cudaSuccess && !th->chem_sampled) e = cudaMalloc(&th->chem_sampled, sizeof(double) * NSPEC * ntiles);
   if (e == cudaSuccess) e = cudaMemset(th->chem_stats, 0, 2 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMemcpy(th->chem_mlp, h, sizeof(DgChemMlp), cudaMemcpyHostToDevice);
   free(h);

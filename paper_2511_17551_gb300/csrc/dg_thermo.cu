@@ -16,6 +16,7 @@
 // residual in double-FP32 pairs.
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include "dg_dd.cuh"
@@ -317,12 +318,15 @@ void dg_thermo_free(DgThermo* th) {
   if (th->chem_mlp) cudaFree(th->chem_mlp);
   if (th->chem_stats) cudaFree(th->chem_stats);
   if (th->chem_flags) cudaFree(th->chem_flags);
+  if (th->chem_sampled) cudaFree(th->chem_sampled);
   if (th->chem_corr) cudaFree(th->chem_corr);
   if (th->chem_trust) cudaFree(th->chem_trust);
   if (th->species) cudaFree(th->species);
   if (th->coef32) cudaFree(th->coef32);
   if (th->species_raw) cudaFree(th->species_raw);
   if (th->reac) cudaFree(th->reac);
+  free(th->chem_tab32);
+  if (th->chem_exp2) cudaFree(th->chem_exp2);
   if (th->src) cudaFree(th->src);
   if (th->T) cudaFree(th->T);
   if (th->pc) cudaFree(th->pc);

@@ -15,6 +15,8 @@ struct DgThermo {
   unsigned long long* status;
   double* species_raw; // device [ns][16] chemistry coefficient rows (dg_chem.cu)
   double* reac;        // device [nr][20] reaction rows (ln A in slot 16)
+  void* chem_tab32;    // host: the same rows as double-FP32 pairs, a kernel argument (dg_chem.cu)
+  void* chem_exp2;     // device: 2^(j/128) as pairs
   int nr;              // number of reactions, 0 = frozen
   void* src;           // device [K][ns][np] chemistry source (form precision)
   void* mlp;           // temperature surrogate weights (device) or null
@@ -22,6 +24,7 @@ struct DgThermo {
   void* chem_mlp;                 // chemistry-source surrogate (device) or null
   unsigned long long* chem_stats; // [accepted, fallback] node counts of the source surrogate
   unsigned char* chem_flags;      // per 32-node tile: 0 accepted, otherwise recomputed plainly
+  void* chem_sampled;             // [tiles][5] (form precision): the plain source at each tile's sampled node
   unsigned long long chem_calls;  // learned-source evaluations so far (moves each tile's sampled node)
   int src_valid;                  // src holds an evaluation
   float* chem_corr;               // [10][K np] plain-minus-network corrections of the learned source
