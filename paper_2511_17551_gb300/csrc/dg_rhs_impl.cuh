@@ -4,9 +4,12 @@
 //
 // The right-hand-side kernel comes in three flavours: FL = 1 fixes the production flux
 // pair at compile time (Ranocha volume flux for one gas, Ducros for mixtures; LLF at
-// interfaces and subcells, constant viscosity), FL = 2 + vf fixes another one-gas volume
+// interfaces and subcells), FL = 2 + vf fixes another one-gas volume
 // flux vf with LLF and constant viscosity (the split forms, emitted for 3D at N = 3), and
-// FL = 0 switches on the runtime choice (every other pair, and Sutherland's law).
+// FL = 0 switches on the runtime choice (every other pair).  Sutherland's law touches this kernel
+// only in the wave speeds of a step's last stage and at inflow faces: FL = 1 carries it by a test
+// of its constant (the same registers and spills; 16^3 elements, N = 7, 417 us a stage in the
+// runtime-choice kernel, 219 here; the pair without it 124 us at 32^3, N = 3, either way).
 // A translation unit that defines DG_GENERIC_ONLY emits only the FL = 0 kernels (and
 // its own basis table); one that also defines DG_SPLIT_ONLY emits only the FL = 2 + vf
 // kernels; the main one emits everything else and forwards the other pairs to
@@ -668,7 +671,7 @@ rhs_kernel(const DgArgs a, const KConst kc) {
             fx[DIM] = bkind == DG_BC_ISOTHERMAL ? h : real(0);
           } else {  // inflow
             real r = 1;
-            if (!FL && kc.suth_s > real(0))
+            if (FL < 2 && kc.suth_s > real(0))
               r = sutherland_ratio(x.p * RealOps<real>::rcp(x.rho), kc.suth_s, kc.suth_c1, kc.suth_irt) *
                   RealOps<real>::rcp(sutherland_ratio(o.p * RealOps<real>::rcp(o.rho), kc.suth_s, kc.suth_c1,
                                                       kc.suth_irt));
@@ -905,7 +908,7 @@ rhs_kernel(const DgArgs a, const KConst kc) {
         }
         la *= ij;
         lv *= ij * ij * kc.visc * ir;
-        if (!FL && kc.suth_s > real(0)) lv *= sutherland_ratio(p * ir, kc.suth_s, kc.suth_c1, kc.suth_irt);
+        if (FL < 2 && kc.suth_s > real(0)) lv *= sutherland_ratio(p * ir, kc.suth_s, kc.suth_c1, kc.suth_irt);
         if (!(p > real(0)) || !isfinite(la)) {
           latch_status(a.status, DG_ST_NONPHYS, e0 + e);
           la = real(0);
@@ -1840,8 +1843,7 @@ cudaError_t DG_CAT(DG_PREFIX, _rhs)(const DgArgs& a, cudaStream_t st) {
 #else
 cudaError_t DG_CAT(DG_PREFIX, _rhs)(const DgArgs& a, cudaStream_t st) {
 #ifndef DG_GENERIC_ONLY
-  const bool production = a.sf == DG_SF_LLF && a.vf == (a.nsp == 1 ? DG_VF_RANOCHA : DG_VF_DUCROS) &&
-                          !(a.suth_s > 0.0);
+  const bool production = a.sf == DG_SF_LLF && a.vf == (a.nsp == 1 ? DG_VF_RANOCHA : DG_VF_DUCROS);
 #ifdef DG_SPLIT_RHS
   const bool split = a.dim == 3 && a.nsp == 1 && a.N == 3 && a.sf == DG_SF_LLF && !(a.suth_s > 0.0) &&
                      a.vf != DG_VF_RANOCHA;
