@@ -68,7 +68,6 @@ struct dg_ctx {
 namespace {
 
 __constant__ double c_D64[(DG_MAXN + 1) * (DG_MAXN + 1)];
-__constant__ double c_w64[DG_MAXN + 1];
 int g_basis_uploaded_for = -1;  // device id
 
 #define CK(x)                                   \
@@ -89,12 +88,9 @@ cudaError_t upload_all_bases(int dev) {
 cudaError_t upload_local_basis(int N) {
   DgHostBasis b;
   if (dg_host_basis(N, &b)) return cudaErrorInvalidValue;
-  double D[(DG_MAXN + 1) * (DG_MAXN + 1)] = {0}, w[DG_MAXN + 1] = {0};
+  double D[(DG_MAXN + 1) * (DG_MAXN + 1)] = {0};
   for (int i = 0; i < (N + 1) * (N + 1); ++i) D[i] = b.D[i];
-  for (int i = 0; i <= N; ++i) w[i] = b.w[i];
-  cudaError_t e = cudaMemcpyToSymbol(c_D64, D, sizeof(D));
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_w64, w, sizeof(w));
-  return e;
+  return cudaMemcpyToSymbol(c_D64, D, sizeof(D));
 }
 
 __device__ __forceinline__ int ipow_d(int b, int e) {
@@ -292,89 +288,139 @@ __global__ void prim2cons_kernel(const double* w, T* u, float* lo, int64_t K, in
   }
 }
 
-// FP64 domain integrals, per block partial sums (deterministic: fixed order later)
-template <typename T>
-__global__ void diag_kernel(const T* u, const double* Ja, const double* J, int64_t K, int dim,
-                            int N, int nsp, double gamma, int single_gas, double suth_s,
-                            double suth_rt, double* partial) {
-  const int np = ipow_d(N + 1, dim), nv = nsp + dim + 1;
+// FP64 domain integrals, per block partial sums (deterministic: the grid depends on K alone, fixed
+// order within a block and over the blocks).  A CTA takes EPB elements at a time: the velocities
+// of their nodes go to shared memory in FP64, then each thread forms its nodes' derivative sums
+// from there.  What bounds it is the FP64 pipe (about 170 operations a node at N = 3, 50 of them
+// the two logarithms); with every thread forming its neighbours' velocities from the global state
+// and sums in local memory it took 378 us a call at 8^3 and 3.5 ms at 32^3 elements, N = 3, now
+// 60 us and 0.83 ms.  The basis comes by value: two copies to a constant symbol per call, shared by
+// the contexts of a process, took 15 us of a call.
+struct DiagBasis {
+  double D[(DG_MAXN + 1) * (DG_MAXN + 1)], w[DG_MAXN + 1];
+};
+constexpr int DIAG_TPB = 256;
+
+template <typename T, int DIM, int N>
+__global__ void __launch_bounds__(DIAG_TPB) diag_kernel(const T* u, const double* Ja, const double* J, int64_t K,
+                                                        int nsp, double gamma, int single_gas, double suth_s,
+                                                        double suth_rt, const __grid_constant__ DiagBasis B,
+                                                        double* partial) {
+  constexpr int N1 = N + 1, NP = DIM == 3 ? N1 * N1 * N1 : N1 * N1;
+  constexpr int EPB = NP >= DIAG_TPB ? 1 : DIAG_TPB / NP;
+  __shared__ double sv[EPB][DIM][NP];
+  __shared__ double sD[N1 * N1], sw[N1];
+  const int tid = threadIdx.x, nv = nsp + DIM + 1;
+  if (tid < N1 * N1) sD[tid] = B.D[tid];
+  if (tid < N1) sw[tid] = B.w[tid];
   double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < K * np;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t k = i / np;
-    const int node = (int)(i % np);
-    const T* uu = u + k * nv * np;
-    double wq = 1.0;
-    for (int d = 0; d < dim; ++d) wq *= c_w64[(node / ipow_d(N + 1, d)) % (N + 1)];
-    const double Jn = J[k * np + node];
-    double rho = 0.0;
-    for (int s = 0; s < nsp; ++s) rho += (double)uu[s * np + node];
-    double v[3] = {0, 0, 0}, v2 = 0.0;
-    for (int d = 0; d < dim; ++d) {
-      v[d] = (double)uu[(nsp + d) * np + node] / rho;
-      v2 += v[d] * v[d];
+  for (int64_t e0 = blockIdx.x * (int64_t)EPB; e0 < K; e0 += gridDim.x * (int64_t)EPB) {
+    const int ne = (int)((K - e0) < EPB ? (K - e0) : EPB);
+    __syncthreads();  // the previous group's velocities are read
+    for (int i = tid; i < ne * NP; i += DIAG_TPB) {
+      const int e = i / NP, node = i % NP;
+      const T* uu = u + (e0 + e) * nv * NP + node;
+      double rho = 0.0;
+      for (int s = 0; s < nsp; ++s) rho += (double)uu[s * NP];
+      const double ir = 1.0 / rho;
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) sv[e][d][node] = (double)uu[(nsp + d) * NP] * ir;
     }
-    const double rhoE = (double)uu[(nsp + dim) * np + node];
-    double gv[3][3] = {{0}};
-    const int n1 = N + 1;
-    for (int a = 0; a < dim; ++a)
-      for (int d = 0; d < dim; ++d) {
-        const int s = ipow_d(n1, d), pos = (node / s) % n1, base = node - pos * s;
-        double dv = 0.0;
-        for (int l = 0; l < n1; ++l) {
-          const int m = base + l * s;
-          double rm = 0.0;
-          for (int q = 0; q < nsp; ++q) rm += (double)uu[q * np + m];
-          dv += c_D64[pos * n1 + l] * ((double)uu[(nsp + a) * np + m] / rm);
-        }
-        for (int x = 0; x < dim; ++x) gv[a][x] += Ja[((k * dim + d) * dim + x) * np + node] * dv / Jn;
-      }
-    double w2;
-    if (dim == 3) {
-      double wx = gv[2][1] - gv[1][2], wy = gv[0][2] - gv[2][0], wz = gv[1][0] - gv[0][1];
-      w2 = wx * wx + wy * wy + wz * wz;
-    } else {
-      double wz = gv[1][0] - gv[0][1];
-      w2 = wz * wz;
-    }
-    double div = 0.0;
-    for (int a = 0; a < dim; ++a) div += gv[a][a];
-    const double dV = wq * Jn;
-    acc[0] += dV;
-    acc[1] += dV * 0.5 * rho * v2;
-    acc[2] += dV * 0.5 * rho * w2;
-    if (single_gas) {
-      double p = (gamma - 1.0) * (rhoE - 0.5 * rho * v2);
-      acc[3] += dV * (-rho * (log(p) - gamma * log(rho)) / (gamma - 1.0));
-    }
-    acc[4] += dV * rho;
-    acc[5] += dV * rhoE;
-    // Sutherland weight mu(T)/mu of the dissipation integrals (Eqs. TGV_SD, TGV_DD)
-    double mr = 1.0;
-    if (single_gas && suth_s > 0.0) {
-      const double th = (gamma - 1.0) * (rhoE - 0.5 * rho * v2) / (rho * suth_rt);
-      mr = (1.0 + suth_s) * th * sqrt(th) / (th + suth_s);
-    }
-    acc[6] += dV * mr * div * div;
-    acc[7] += dV * mr * w2;
-  }
-  __shared__ double red[8][256];
-  for (int q = 0; q < 8; ++q) red[q][threadIdx.x] = acc[q];
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w)
-      for (int q = 0; q < 8; ++q) red[q][threadIdx.x] += red[q][threadIdx.x + w];
     __syncthreads();
+    for (int i = tid; i < ne * NP; i += DIAG_TPB) {
+      const int e = i / NP, node = i % NP;
+      const int64_t k = e0 + e;
+      const T* uu = u + k * nv * NP + node;
+      const int pos[3] = {node % N1, (node / N1) % N1, DIM == 3 ? node / (N1 * N1) : 0};
+      double wq = sw[pos[0]] * sw[pos[1]];
+      if (DIM == 3) wq *= sw[pos[2]];
+      const double Jn = J[k * NP + node], iJ = 1.0 / Jn;
+      double rho = 0.0;
+      for (int s = 0; s < nsp; ++s) rho += (double)uu[s * NP];
+      const double rhoE = (double)uu[(nsp + DIM) * NP];
+      double v2 = 0.0, dv[DIM][DIM];  // dv[a][d] = d v_a / d xi_d
+#pragma unroll
+      for (int a = 0; a < DIM; ++a) {
+        v2 += sv[e][a][node] * sv[e][a][node];
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) {
+          const int st = d == 0 ? 1 : (d == 1 ? N1 : N1 * N1), base = node - pos[d] * st;
+          double x = 0.0;
+#pragma unroll
+          for (int l = 0; l < N1; ++l) x += sD[pos[d] * N1 + l] * sv[e][a][base + l * st];
+          dv[a][d] = x;
+        }
+      }
+      double gv[DIM][DIM];  // d v_a / d x_x
+#pragma unroll
+      for (int x = 0; x < DIM; ++x) {
+        double ja[DIM];
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) ja[d] = Ja[((k * DIM + d) * DIM + x) * NP + node] * iJ;
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+          double g = 0.0;
+#pragma unroll
+          for (int d = 0; d < DIM; ++d) g += ja[d] * dv[a][d];
+          gv[a][x] = g;
+        }
+      }
+      double w2, div = 0.0;
+      const double wz = gv[1][0] - gv[0][1];
+      if (DIM == 3) {
+        const double wx = gv[DIM - 1][1] - gv[1][DIM - 1], wy = gv[0][DIM - 1] - gv[DIM - 1][0];
+        w2 = wx * wx + wy * wy + wz * wz;
+      } else {
+        w2 = wz * wz;
+      }
+#pragma unroll
+      for (int a = 0; a < DIM; ++a) div += gv[a][a];
+      const double dV = wq * Jn;
+      acc[0] += dV;
+      acc[1] += dV * 0.5 * rho * v2;
+      acc[2] += dV * 0.5 * rho * w2;
+      // Sutherland weight mu(T)/mu of the dissipation integrals (Eqs. TGV_SD, TGV_DD)
+      double mr = 1.0;
+      if (single_gas) {
+        const double p = (gamma - 1.0) * (rhoE - 0.5 * rho * v2);
+        acc[3] += dV * (-rho * (log(p) - gamma * log(rho)) / (gamma - 1.0));
+        if (suth_s > 0.0) {
+          const double th = p / (rho * suth_rt);
+          mr = (1.0 + suth_s) * th * sqrt(th) / (th + suth_s);
+        }
+      }
+      acc[4] += dV * rho;
+      acc[5] += dV * rhoE;
+      acc[6] += dV * mr * div * div;
+      acc[7] += dV * mr * w2;
+    }
   }
-  if (threadIdx.x == 0)
-    for (int q = 0; q < 8; ++q) partial[blockIdx.x * 8 + q] = red[q][0];
+  __shared__ double red[DIAG_TPB / 32][8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+    if ((tid & 31) == 0) red[tid >> 5][q] = acc[q];
+  }
+  __syncthreads();
+  if (tid < 8) {
+    double x = 0.0;
+    for (int i = 0; i < DIAG_TPB / 32; ++i) x += red[i][tid];
+    partial[blockIdx.x * 8 + tid] = x;
+  }
 }
 
-__global__ void diag_final_kernel(const double* partial, int nb, double* out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int b = 0; b < nb; ++b)
-    for (int q = 0; q < 8; ++q) s[q] += partial[b * 8 + q];
+// one warp per integral: the block sums in a fixed order
+__global__ void __launch_bounds__(256) diag_final_kernel(const double* partial, int nb, double* out) {
+  __shared__ double s[8];
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double x = 0.0;
+  for (int b = lane; b < nb; b += 32) x += partial[b * 8 + q];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  if (lane == 0) s[q] = x;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   out[0] = s[1] / s[0];
   out[1] = s[2] / s[0];
   out[2] = s[3];
@@ -383,6 +429,25 @@ __global__ void diag_final_kernel(const double* partial, int nb, double* out) {
   out[5] = s[0];
   out[6] = s[6] / s[0];
   out[7] = s[7] / s[0];
+}
+
+template <typename T, int DIM>
+cudaError_t launch_diag(dg_ctx* c, const DiagBasis& B, int max_blocks, int* blocks) {
+  const T* u = (const T*)c->u[c->cur];
+  const int64_t per = c->np >= DIAG_TPB ? 1 : DIAG_TPB / c->np, groups = (c->K + per - 1) / per;
+  const int nb = *blocks = (int)(groups < max_blocks ? groups : max_blocks);
+#define DG_DIAG(N)                                                                                              \
+  diag_kernel<T, DIM, N><<<nb, DIAG_TPB, 0, c->stream>>>(u, c->Ja64, c->J64, c->K, c->nsp, c->gamma,            \
+                                                         c->n_species == 0, c->suth_s, c->suth_rt, B, c->partial)
+  switch (c->N) {
+    case 2: DG_DIAG(2); break;
+    case 3: DG_DIAG(3); break;
+    case 4: DG_DIAG(4); break;
+    case 7: DG_DIAG(7); break;
+    default: return cudaErrorInvalidValue;
+  }
+#undef DG_DIAG
+  return cudaGetLastError();
 }
 
 void rk_ck45(double* A, double* B) {
@@ -1053,19 +1118,20 @@ dg_status dg_diagnostics(dg_ctx* c, double out[8]) {
   if (!c || !out) return DG_EINVAL;
   if (!c->have_state) return DG_ESTATE;
   cudaSetDevice(c->dev);
-  CK(upload_local_basis(c->N));
+  DiagBasis B;
+  DgHostBasis hb;
+  if (dg_host_basis(c->N, &hb)) return DG_EINVAL;
+  memset(&B, 0, sizeof(B));
+  memcpy(B.D, hb.D, sizeof(double) * (c->N + 1) * (c->N + 1));
+  memcpy(B.w, hb.w, sizeof(double) * (c->N + 1));
   double* dout = c->partial;  // reuse the tail of the partial buffer for the result
-  const int nb = c->diag_blocks - 2;
+  const int most = c->diag_blocks - 2;
+  int nb = 0;
   if (c->precision == DG_MIXED)
-    diag_kernel<float><<<nb, 256, 0, c->stream>>>((const float*)c->u[c->cur], c->Ja64, c->J64,
-                                                  c->K, c->dim, c->N, c->nsp, c->gamma,
-                                                  c->n_species == 0, c->suth_s, c->suth_rt, c->partial);
+    CK((c->dim == 3 ? launch_diag<float, 3>(c, B, most, &nb) : launch_diag<float, 2>(c, B, most, &nb)));
   else
-    diag_kernel<double><<<nb, 256, 0, c->stream>>>((const double*)c->u[c->cur], c->Ja64, c->J64,
-                                                   c->K, c->dim, c->N, c->nsp, c->gamma,
-                                                   c->n_species == 0, c->suth_s, c->suth_rt, c->partial);
-  CK(cudaGetLastError());
-  diag_final_kernel<<<1, 32, 0, c->stream>>>(c->partial, nb, dout + nb * 8);
+    CK((c->dim == 3 ? launch_diag<double, 3>(c, B, most, &nb) : launch_diag<double, 2>(c, B, most, &nb)));
+  diag_final_kernel<<<1, 256, 0, c->stream>>>(c->partial, nb, dout + nb * 8);
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(out, dout + nb * 8, sizeof(double) * 8, cudaMemcpyDeviceToHost, c->stream));
   dg_status w = wait_stream(c);
