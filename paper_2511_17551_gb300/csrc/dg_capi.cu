@@ -263,29 +263,44 @@ void launch_merge(const float* hi, const float* lo, double* dst, int64_t n, cuda
   }
 }
 
-// one-gas primitive (rho, v, p) -> conserved, written in the form precision
-// (lo: the FP32 form's compensation part, or null)
-template <typename T>
-__global__ void prim2cons_kernel(const double* w, T* u, float* lo, int64_t K, int dim, int np, double gamma) {
-  const int nv = dim + 2;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < K * np;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t k = i / np;
-    const int node = (int)(i % np);
-    const double* ww = w + k * nv * np + node;
-    T* uu = u + k * nv * np + node;
-    double rho = ww[0], ke = 0.0, c[8];
-    c[0] = rho;
-    for (int d = 0; d < dim; ++d) {
-      c[1 + d] = rho * ww[(1 + d) * np];
-      ke += ww[(1 + d) * np] * ww[(1 + d) * np];
+// one-gas primitive (rho, v, p) -> conserved, written in the form precision (lo: the FP32 form's
+// compensation part, or null).  Bound by memory: (dim + 2) doubles in, as many bytes out.  The values
+// stay in registers (compile-time dim; with a run-time one they went through local memory), and
+// the 64-bit division that splits the node index is one per CTA and pass: 32^3 elements, N = 3,
+// a call 162 -> 147 us (the conversions of the hi / lo split on the FP64 pipe are what is left).
+template <typename T, int DIM>
+__global__ void __launch_bounds__(256) prim2cons_kernel(const double* w, T* u, float* lo, int64_t K, int np,
+                                                        double gamma) {
+  constexpr int NV = DIM + 2;
+  const double igm1 = 1.0 / (gamma - 1.0);
+  for (int64_t base = blockIdx.x * (int64_t)256; base < K * np; base += gridDim.x * (int64_t)256) {
+    const int64_t k0 = base / np;
+    const unsigned off = (unsigned)(base - k0 * np) + threadIdx.x, dk = off / (unsigned)np;
+    const int64_t k = k0 + dk;
+    if (k >= K) continue;
+    const int64_t at = k * NV * np + (off - dk * (unsigned)np);
+    double c[NV], ke = 0.0;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) c[v] = w[at + v * np];
+#pragma unroll
+    for (int d = 1; d <= DIM; ++d) {
+      ke += c[d] * c[d];
+      c[d] *= c[0];
     }
-    c[1 + dim] = ww[(1 + dim) * np] / (gamma - 1.0) + 0.5 * rho * ke;
-    for (int v = 0; v < nv; ++v) {
-      uu[v * np] = (T)c[v];
-      if (lo) lo[k * nv * np + v * np + node] = (float)(c[v] - (double)(T)c[v]);
+    c[1 + DIM] = c[1 + DIM] * igm1 + 0.5 * c[0] * ke;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const T h = (T)c[v];
+      u[at + v * np] = h;
+      if (lo) lo[at + v * np] = (float)(c[v] - (double)h);
     }
   }
+}
+template <typename T>
+void launch_prim2cons(const double* w, T* u, float* lo, int64_t K, int dim, int np, double gamma, unsigned grid,
+                      cudaStream_t st) {
+  if (dim == 3) prim2cons_kernel<T, 3><<<grid, 256, 0, st>>>(w, u, lo, K, np, gamma);
+  else prim2cons_kernel<T, 2><<<grid, 256, 0, st>>>(w, u, lo, K, np, gamma);
 }
 
 // FP64 domain integrals, per block partial sums (deterministic: the grid depends on K alone, fixed
@@ -909,9 +924,9 @@ dg_status dg_init_mesh(const dg_mesh_desc* m, const dg_physics_desc* p, dg_ctx**
       cudaError_t e2;
       if (c->n_species == 0) {
         if (c->precision == DG_MIXED)
-          prim2cons_kernel<float><<<1, 32, 0, c->stream>>>(bw, (float*)c->bc_u, NULL, p->n_bc, dim, 1, c->gamma);
+          launch_prim2cons<float>(bw, (float*)c->bc_u, NULL, p->n_bc, dim, 1, c->gamma, 1, c->stream);
         else
-          prim2cons_kernel<double><<<1, 32, 0, c->stream>>>(bw, (double*)c->bc_u, NULL, p->n_bc, dim, 1, c->gamma);
+          launch_prim2cons<double>(bw, (double*)c->bc_u, NULL, p->n_bc, dim, 1, c->gamma, 1, c->stream);
         e2 = cudaGetLastError();
       } else {
         e2 = dg_thermo_boundary(&c->th, bw, p->n_bc, c->bc_u, c->stream);
@@ -984,11 +999,11 @@ dg_status dg_set_state_primitive(dg_ctx* c, const double* w, int on_device, doub
   }
   if (c->n_species == 0) {
     if (c->precision == DG_MIXED)
-      prim2cons_kernel<float><<<grid_for(c->K * c->np, 256), 256, 0, c->stream>>>(
-          src, (float*)c->u[c->cur], c->ulo, c->K, c->dim, c->np, c->gamma);
+      launch_prim2cons<float>(src, (float*)c->u[c->cur], c->ulo, c->K, c->dim, c->np, c->gamma,
+                              grid_for(c->K * c->np, 256), c->stream);
     else
-      prim2cons_kernel<double><<<grid_for(c->K * c->np, 256), 256, 0, c->stream>>>(
-          src, (double*)c->u[c->cur], NULL, c->K, c->dim, c->np, c->gamma);
+      launch_prim2cons<double>(src, (double*)c->u[c->cur], NULL, c->K, c->dim, c->np, c->gamma,
+                               grid_for(c->K * c->np, 256), c->stream);
     CK(cudaGetLastError());
   } else {
     // also seeds the temperature cache with the given temperatures; the compensation part
