@@ -269,126 +269,238 @@ __global__ void mlp_forward_f32_kernel(const float* P, int no, const float* X, f
 #define OFF_B1 (NH * NI)
 #define OFF_W2 (OFF_B1 + NH)
 #define OFF_B2 (OFF_W2 + NH * NH)
-struct TrainSmem {
-  float W1[NH * NI], b1[NH], W2[NH * NH], W2T[NH * NH], b2[NH], W3[NO_MAX * NH], b3[NO_MAX];
-  float X[TS][NI], a1[TS][NH], h1[TS][NH], a2[TS][NH], h2[TS][NH];
+constexpr int TT = 256;        // threads of a training CTA
+constexpr int HP = NH + 4;     // padded row of a [sample][unit] array: float4 rows on distinct banks
+constexpr int XP = NI + 1;     // features and a constant 1 (the bias column of layer 1's gradient)
+struct __align__(16) TrainSmem {
+  float W2[NH][NH], W2T[NH][HP];  // [j][i], [i][j]
+  float W3[NO_MAX][HP];
+  float h1[TS][HP], e1[TS][HP], h2[TS][HP], e2[TS][HP];  // activations, and GELU's derivative (e2: delta 2)
+  float W1[NH][XP], b2[NH], b3[NO_MAX], X[TS][XP];
   float dy[TS][NO_MAX], r2[TS][NO_MAX];
-  float g[dg_mlp_np(NO_MAX)];  // gW2 stored transposed [i][j]
-  float loss;
 };
 
+// GELU and its derivative from one tanh
+__device__ __forceinline__ void gelu_and_d(float x, float& g, float& d) {
+  const float k = 0.7978845608028654f;
+  const float t = tanhf(k * (x + 0.044715f * x * x * x));
+  g = 0.5f * x * (1.0f + t);
+  d = 0.5f * (1.0f + t) + 0.5f * x * (1.0f - t * t) * k * (1.0f + 3.0f * 0.044715f * x * x);
+}
+
+// acc[r][c] += sum over q of a[row r][q] b[q][col c] for this thread's 2 rows and 4 columns
+// (a [.][HP], b [NH][LD])
+template <int LD>
+__device__ __forceinline__ void tile_2x4(const float* a0, const float* a1, const float* b, float (*acc)[4]) {
+#pragma unroll 4
+  for (int q = 0; q < NH; q += 4) {
+    const float4 u = *reinterpret_cast<const float4*>(a0 + q), v = *reinterpret_cast<const float4*>(a1 + q);
+    const float x0[4] = {u.x, u.y, u.z, u.w}, x1[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const float4 w = *reinterpret_cast<const float4*>(b + (q + r) * LD);
+      acc[0][0] += x0[r] * w.x; acc[0][1] += x0[r] * w.y; acc[0][2] += x0[r] * w.z; acc[0][3] += x0[r] * w.w;
+      acc[1][0] += x1[r] * w.x; acc[1][1] += x1[r] * w.y; acc[1][2] += x1[r] * w.z; acc[1][3] += x1[r] * w.w;
+    }
+  }
+}
+
 // per-CTA partial gradients of loss = (1/(B no)) sum_s sum_o (y_so - t_so)^2 over the
-// CTA's tiles
-__global__ void __launch_bounds__(NH) mlp_grad_kernel(const float* P, int no, const float* X, const float* t,
-                                                      int B, float* partial) {
+// CTA's tiles of TS samples, summed in a fixed order.  The three 64-wide products of a tile (layer 2,
+// its transpose, its gradient) are 2 x 4 and 4 x 4 register tiles over 256 threads with 16-byte
+// shared-memory reads; the gradient sums stay in registers over the tiles.  With 64 threads, one
+// per unit, and every operand read 4 bytes at a time, a fitting iteration (two
+// gathers, this, Adam) with a batch of 4,096 and ten outputs took 88 us, now 36; what is left is the
+// chain of eight barriers of one tile per CTA (128 CTAs) and the launches.
+__global__ void __launch_bounds__(TT) mlp_grad_kernel(const float* P, int no, const float* X, const float* t, int B,
+                                                      float* partial) {
   extern __shared__ __align__(16) unsigned char raw[];
   TrainSmem& S = *reinterpret_cast<TrainSmem*>(raw);
-  const int j = threadIdx.x;
+  const int tid = threadIdx.x;
   const int OW3 = dg_mlp_off_w3(), OB3 = dg_mlp_off_b3(no), NPAR = dg_mlp_np(no);
-  for (int q = j; q < NH * NI; q += NH) S.W1[q] = P[OFF_W1 + q];
-  for (int q = j; q < NH * NH; q += NH) {
-    S.W2[q] = P[OFF_W2 + q];
-    S.W2T[(q % NH) * NH + q / NH] = P[OFF_W2 + q];
+#pragma unroll 4
+  for (int q = tid; q < NH * NH; q += TT) {
+    const float w = P[OFF_W2 + q];
+    S.W2[q / NH][q % NH] = w;
+    S.W2T[q % NH][q / NH] = w;
   }
-  S.b1[j] = P[OFF_B1 + j];
-  S.b2[j] = P[OFF_B2 + j];
-  for (int o = 0; o < no; ++o) S.W3[o * NH + j] = P[OW3 + o * NH + j];
-  if (j < no) S.b3[j] = P[OB3 + j];
-  if (j == 0) S.loss = 0.f;
-  for (int q = j; q < NPAR; q += NH) S.g[q] = 0.f;
-  __syncthreads();
+  for (int q = tid; q < NH * NI; q += TT) S.W1[q / NI][q % NI] = P[OFF_W1 + q];
+  if (tid < NH) {
+    S.W1[tid][NI] = P[OFF_B1 + tid];
+    S.b2[tid] = P[OFF_B2 + tid];
+  }
+  for (int q = tid; q < no * NH; q += TT) S.W3[q / NH][q % NH] = P[OW3 + q];
+  if (tid < no) S.b3[tid] = P[OB3 + tid];
   const float inv = 1.0f / ((float)B * (float)no);
+  // thread roles: unit j of the one-unit passes with 8 samples from s8; columns 4 c4 of the tiled
+  // passes with rows 2 r2 (samples) or 4 r2 (units)
+  const int j = tid & (NH - 1), s8 = (tid >> 6) * 8, c4 = (tid & 15) * 4, rw = tid >> 4;
+  float gW2[4][4] = {}, gW3[NO_MAX / 4] = {}, gW1[2] = {0.f, 0.f}, gb2 = 0.f, gb3 = 0.f, loss = 0.f;
   for (int s0 = blockIdx.x * TS; s0 < B; s0 += gridDim.x * TS) {
     const int ns = min(TS, B - s0);
-    for (int q = j; q < TS * NI; q += NH) S.X[q / NI][q % NI] = q / NI < ns ? X[(int64_t)s0 * NI + q] : 0.f;
+    // samples past the batch: zero features, and zero dy below, add nothing
+    for (int q = tid; q < TS * XP; q += TT) {
+      const int s = q / XP, k = q % XP;
+      S.X[s][k] = k == NI ? 1.0f : (s < ns ? X[(int64_t)(s0 + s) * NI + k] : 0.0f);
+    }
     __syncthreads();
-    for (int s = 0; s < ns; ++s) {
-      float a = S.b1[j];
+#pragma unroll 2
+    for (int s = s8; s < s8 + 8; ++s) {
+      float a = S.W1[j][NI];
 #pragma unroll
-      for (int k = 0; k < NI; ++k) a += S.W1[j * NI + k] * S.X[s][k];
-      S.a1[s][j] = a;
-      S.h1[s][j] = gelu_f(a);
+      for (int k = 0; k < NI; ++k) a += S.W1[j][k] * S.X[s][k];
+      gelu_and_d(a, S.h1[s][j], S.e1[s][j]);
     }
     __syncthreads();
-    for (int s = 0; s < ns; ++s) {
-      float a = S.b2[j];
-      for (int i = 0; i < NH; ++i) a += S.W2T[i * NH + j] * S.h1[s][i];
-      S.a2[s][j] = a;
-      S.h2[s][j] = gelu_f(a);
+    {
+      float acc[2][4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[0][c] = acc[1][c] = S.b2[c4 + c];
+      tile_2x4<HP>(S.h1[2 * rw], S.h1[2 * rw + 1], &S.W2T[0][c4], acc);
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) gelu_and_d(acc[r][c], S.h2[2 * rw + r][c4 + c], S.e2[2 * rw + r][c4 + c]);
     }
     __syncthreads();
-    for (int q = j; q < ns * no; q += NH) {
+    for (int q = tid; q < TS * no; q += TT) {
       const int s = q / no, o = q % no;
       float y = S.b3[o];
-      for (int i = 0; i < NH; ++i) y += S.W3[o * NH + i] * S.h2[s][i];
-      const float r = y - t[(int64_t)(s0 + s) * no + o];
+#pragma unroll 4
+      for (int i = 0; i < NH; i += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(&S.W3[o][i]);
+        const float4 h = *reinterpret_cast<const float4*>(&S.h2[s][i]);
+        y += w.x * h.x;
+        y += w.y * h.y;
+        y += w.z * h.z;
+        y += w.w * h.w;
+      }
+      const float r = s < ns ? y - t[(int64_t)(s0 + s) * no + o] : 0.0f;
       S.dy[s][o] = 2.0f * r * inv;
       S.r2[s][o] = r * r * inv;
     }
     __syncthreads();
-    if (j == 0)  // fixed order: deterministic
-      for (int s = 0; s < ns; ++s)
-        for (int o = 0; o < no; ++o) S.loss += S.r2[s][o];
-    float gb2 = 0.f;
-    for (int o = 0; o < no; ++o) {
-      float gw3 = 0.f;
-      for (int s = 0; s < ns; ++s) gw3 += S.dy[s][o] * S.h2[s][j];
-      S.g[OW3 + o * NH + j] += gw3;
+    // the output layer's gradients, then delta 2 in place of GELU's derivative
+#pragma unroll
+    for (int m = 0; m < NO_MAX / 4; ++m) {
+      const int o = (tid >> 6) + 4 * m;
+      if (o < no) {
+        float g = 0.f;
+#pragma unroll 8
+        for (int s = 0; s < TS; ++s) g += S.dy[s][o] * S.h2[s][j];
+        gW3[m] += g;
+      }
     }
-    for (int s = 0; s < ns; ++s) {
+    if (tid < no) {
+      float g = 0.f, l = 0.f;
+      for (int s = 0; s < TS; ++s) {
+        g += S.dy[s][tid];
+        l += S.r2[s][tid];
+      }
+      gb3 += g;
+      loss += l;
+    }
+#pragma unroll 2
+    for (int s = s8; s < s8 + 8; ++s) {
       float back = 0.f;
-      for (int o = 0; o < no; ++o) back += S.dy[s][o] * S.W3[o * NH + j];
-      const float d2 = back * gelu_d_f(S.a2[s][j]);
-      S.a2[s][j] = d2;  // a2 now holds delta2
-      gb2 += d2;
-    }
-    S.g[OFF_B2 + j] += gb2;
-    if (j < no) {
-      float gb3 = 0.f;
-      for (int s = 0; s < ns; ++s) gb3 += S.dy[s][j];
-      S.g[OB3 + j] += gb3;
+      for (int o = 0; o < no; ++o) back += S.dy[s][o] * S.W3[o][j];
+      S.e2[s][j] *= back;
     }
     __syncthreads();
-    // thread j: row j of dW2 (stored transposed) and delta1 of hidden unit j
-    for (int i = 0; i < NH; ++i) {
-      float acc = 0.f;
-      for (int s = 0; s < ns; ++s) acc += S.a2[s][j] * S.h1[s][i];
-      S.g[OFF_W2 + i * NH + j] += acc;
-    }
-    float gb1 = 0.f, gw1[NI] = {0, 0, 0, 0, 0, 0, 0};
-    for (int s = 0; s < ns; ++s) {
-      float acc = 0.f;
-      for (int q = 0; q < NH; ++q) acc += S.W2[q * NH + j] * S.a2[s][q];
-      const float d1 = acc * gelu_d_f(S.a1[s][j]);
-      gb1 += d1;
+    // layer 2's gradient (units 4 rw.. x inputs c4..)
+    {
+      float g[4][4] = {};
+#pragma unroll 4
+      for (int s = 0; s < TS; ++s) {
+        const float4 d = *reinterpret_cast<const float4*>(&S.e2[s][4 * rw]);
+        const float4 h = *reinterpret_cast<const float4*>(&S.h1[s][c4]);
+        const float dd[4] = {d.x, d.y, d.z, d.w};
 #pragma unroll
-      for (int k = 0; k < NI; ++k) gw1[k] += d1 * S.X[s][k];
-    }
-    S.g[OFF_B1 + j] += gb1;
+        for (int r = 0; r < 4; ++r) {
+          g[r][0] += dd[r] * h.x;
+          g[r][1] += dd[r] * h.y;
+          g[r][2] += dd[r] * h.z;
+          g[r][3] += dd[r] * h.w;
+        }
+      }
 #pragma unroll
-    for (int k = 0; k < NI; ++k) S.g[OFF_W1 + j * NI + k] += gw1[k];
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) gW2[r][c] += g[r][c];
+    }
+    if (tid < NH) {
+      float g = 0.f;
+#pragma unroll 8
+      for (int s = 0; s < TS; ++s) g += S.e2[s][tid];
+      gb2 += g;
+    }
+    // delta 1 = (delta 2 W2) gelu'(a1), in place of the derivative
+    {
+      float acc[2][4] = {};
+      tile_2x4<NH>(S.e2[2 * rw], S.e2[2 * rw + 1], &S.W2[0][c4], acc);
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) S.e1[2 * rw + r][c4 + c] *= acc[r][c];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {  // layer 1: unit q / XP, feature q % XP (the last: the bias)
+      const int q = tid + m * TT;
+      float g = 0.f;
+#pragma unroll 8
+      for (int s = 0; s < TS; ++s) g += S.e1[s][q / XP] * S.X[s][q % XP];
+      gW1[m] += g;
+    }
     __syncthreads();
   }
+  static_assert(NH * XP == 2 * TT, "two entries of layer 1's gradient per thread");
   float* out = partial + (int64_t)blockIdx.x * (NPAR + 1);
-  for (int q = j; q < NPAR; q += NH) {
-    if (q >= OFF_W2 && q < OFF_W2 + NH * NH) {  // back to row-major [j][i]
-      const int i = (q - OFF_W2) / NH, jj = (q - OFF_W2) % NH;
-      out[OFF_W2 + jj * NH + i] = S.g[q];
-    } else {
-      out[q] = S.g[q];
-    }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) out[OFF_W2 + (4 * rw + r) * NH + c4 + c] = gW2[r][c];
+#pragma unroll
+  for (int m = 0; m < 2; ++m) {
+    const int q = tid + m * TT, u = q / XP, k = q % XP;
+    out[k == NI ? OFF_B1 + u : OFF_W1 + u * NI + k] = gW1[m];
   }
-  if (j == 0) out[NPAR] = S.loss;
+#pragma unroll
+  for (int m = 0; m < NO_MAX / 4; ++m) {
+    const int o = (tid >> 6) + 4 * m;
+    if (o < no) out[OW3 + o * NH + j] = gW3[m];
+  }
+  if (tid < NH) out[OFF_B2 + tid] = gb2;
+  if (tid < no) {
+    out[OB3 + tid] = gb3;
+    S.r2[0][tid] = loss;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    float l = 0.f;
+    for (int o = 0; o < no; ++o) l += S.r2[0][o];
+    out[NPAR] = l;
+  }
 }
 
-// fixed-order sum of the partial gradients, then (optionally) one Adam step
-__global__ void mlp_reduce_adam_kernel(const float* partial, int nb, int npar, float* grad, float* P, float* mo,
-                                       float* vo, int step, float lr, float b1, float b2, float eps,
-                                       double* loss) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q > npar) return;
+// fixed-order sum of the partial gradients, then (optionally) one Adam step.  A CTA takes 32
+// parameters, eight slices of the partials each, so that a parameter's sum is a chain of nb / 8
+// loads instead of nb.
+__global__ void __launch_bounds__(256) mlp_reduce_adam_kernel(const float* partial, int nb, int npar, float* grad,
+                                                              float* P, float* mo, float* vo, int step, float lr,
+                                                              float b1, float b2, float eps, double* loss) {
+  __shared__ float part[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = blockIdx.x * 32 + lane;
   float s = 0.f;
-  for (int b = 0; b < nb; ++b) s += partial[(int64_t)b * (npar + 1) + q];
+  if (q <= npar) {
+#pragma unroll 8
+    for (int b = w; b < nb; b += 8) s += partial[(int64_t)b * (npar + 1) + q];
+  }
+  part[w][lane] = s;
+  __syncthreads();
+  if (w != 0 || q > npar) return;
+#pragma unroll
+  for (int i = 1; i < 8; ++i) s += part[i][lane];
   if (q == npar) {
     if (loss) *loss = (double)s;
     return;
@@ -575,7 +687,7 @@ static dg_status grad_common(const float* P, int no, const float* X, const float
   if (cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return DG_ECUDA;
-  mlp_grad_kernel<<<nb, NH, smem, st>>>(P, no, X, t, B, ws);
+  mlp_grad_kernel<<<nb, TT, smem, st>>>(P, no, X, t, B, ws);
   if (cudaGetLastError() != cudaSuccess) return DG_ECUDA;
   *nb_out = nb;
   return DG_OK;
@@ -589,7 +701,7 @@ dg_status dg_mlp_grad(const float* params, int n_out, const float* X, const floa
   if (r != DG_OK) return r;
   if (!grad) return DG_EINVAL;
   const int npar = dg_mlp_np(n_out);
-  mlp_reduce_adam_kernel<<<(npar + 1 + 255) / 256, 256, 0, st>>>(workspace, nb, npar, grad, NULL, NULL, NULL, 0,
+  mlp_reduce_adam_kernel<<<(npar + 1 + 31) / 32, 256, 0, st>>>(workspace, nb, npar, grad, NULL, NULL, NULL, 0,
                                                                  0.f, 0.f, 0.f, 0.f, loss);
   return cudaGetLastError() == cudaSuccess ? DG_OK : DG_ECUDA;
 }
@@ -603,7 +715,7 @@ dg_status dg_mlp_train_step(float* params, int n_out, float* m, float* v, const 
   dg_status r = grad_common(params, n_out, X, t, batch, workspace, ws_bytes, st, &nb);
   if (r != DG_OK) return r;
   const int npar = dg_mlp_np(n_out);
-  mlp_reduce_adam_kernel<<<(npar + 1 + 255) / 256, 256, 0, st>>>(workspace, nb, npar, NULL, params, m, v, step,
+  mlp_reduce_adam_kernel<<<(npar + 1 + 31) / 32, 256, 0, st>>>(workspace, nb, npar, NULL, params, m, v, step,
                                                                  lr, 0.9f, 0.999f, 1e-8f, loss);
   return cudaGetLastError() == cudaSuccess ? DG_OK : DG_ECUDA;
 }

@@ -60,12 +60,6 @@ __device__ __forceinline__ float gelu_fast(float x) {
   asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(z));
   return 0.5f * x * (1.0f + t);
 }
-__device__ __forceinline__ float gelu_d_f(float x) {
-  const float k = 0.7978845608028654f;
-  float t = tanhf(k * (x + 0.044715f * x * x * x));
-  return 0.5f * (1.0f + t) + 0.5f * x * (1.0f - t * t) * k * (1.0f + 3.0f * 0.044715f * x * x);
-}
-
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
