@@ -72,6 +72,11 @@ int dg_host_basis(int N, DgHostBasis* b);
 cudaError_t dg_f64g_upload_basis();
 cudaError_t dg_f32g_upload_basis();
 cudaError_t dg_f32s_upload_basis();
+// the production pair with Sutherland's law
+cudaError_t dg_f32v_upload_basis();
+cudaError_t dg_f64v_upload_basis();
+cudaError_t dg_f32v_rhs(const DgArgs& a, cudaStream_t s);
+cudaError_t dg_f64v_rhs(const DgArgs& a, cudaStream_t s);
 cudaError_t dg_f32s_rhs(const DgArgs& a, cudaStream_t s);
 cudaError_t dg_f64g_rhs(const DgArgs& a, cudaStream_t s);
 cudaError_t dg_f32g_rhs(const DgArgs& a, cudaStream_t s);

@@ -5,6 +5,8 @@
 #define DG_PREFIX dg_f32
 #define DG_GENERIC_RHS dg_f32g_rhs
 #define DG_GENERIC_UPLOAD dg_f32g_upload_basis
+#define DG_SUTH_RHS dg_f32v_rhs
+#define DG_SUTH_UPLOAD dg_f32v_upload_basis
 #define DG_SPLIT_RHS dg_f32s_rhs
 #define DG_SPLIT_UPLOAD dg_f32s_upload_basis
 #include <string.h>

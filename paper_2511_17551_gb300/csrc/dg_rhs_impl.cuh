@@ -4,16 +4,16 @@
 //
 // The right-hand-side kernel comes in three flavours: FL = 1 fixes the production flux
 // pair at compile time (Ranocha volume flux for one gas, Ducros for mixtures; LLF at
-// interfaces and subcells), FL = 2 + vf fixes another one-gas volume
+// interfaces and subcells, constant viscosity), FL = -1 the same with Sutherland's law (it touches
+// this kernel only in the wave speeds of a step's last stage and at inflow faces; 16^3 elements,
+// N = 7: 417 us a stage in the runtime-choice kernel, 219 here; carried by FL = 1 itself it cost the
+// constant-viscosity runs 0.5 %), FL = 2 + vf fixes another one-gas volume
 // flux vf with LLF and constant viscosity (the split forms, emitted for 3D at N = 3), and
-// FL = 0 switches on the runtime choice (every other pair).  Sutherland's law touches this kernel
-// only in the wave speeds of a step's last stage and at inflow faces: FL = 1 carries it by a test
-// of its constant (the same registers and spills; 16^3 elements, N = 7, 417 us a stage in the
-// runtime-choice kernel, 219 here; the pair without it 124 us at 32^3, N = 3, either way).
+// FL = 0 switches on the runtime choice (every other pair).
 // A translation unit that defines DG_GENERIC_ONLY emits only the FL = 0 kernels (and
 // its own basis table); one that also defines DG_SPLIT_ONLY emits only the FL = 2 + vf
-// kernels; the main one emits everything else and forwards the other pairs to
-// DG_SPLIT_RHS (where defined) or DG_GENERIC_RHS.  The split keeps register pressure of the
+// kernels, or with DG_SUTH_ONLY the FL = -1 kernels; the main one emits everything else and
+// forwards the other pairs to DG_SPLIT_RHS (where defined), DG_SUTH_RHS or DG_GENERIC_RHS.  The split keeps register pressure of the
 // compile-time kernels free of the unused branches and lets the parts compile in parallel.
 #pragma once
 #include <stdint.h>
@@ -29,6 +29,10 @@ namespace DG_PREFIX {
 
 using real = DG_REAL;
 using namespace dgk;
+
+// whether the kernel flavour FL fixes the production flux pair
+template <int FL>
+constexpr bool production_pair = FL == 1 || FL == -1;
 
 __constant__ BasisTab<real> c_tab[DG_MAXN + 1];
 
@@ -324,13 +328,13 @@ template <int DIM, int N, int NSP, bool NS, int FL, bool BND = true>
 // (up to 136 registers a thread at 96 threads) instead of 8, so that it does not spill;
 // the split forms (FL >= 2) hold both nodes' conserved states per flux pair: at most 6
 // (96 registers; at 7 the allocator is held to 80 and spills)
-__global__ void __launch_bounds__(Layout<DIM, N, NSP, NS, FL == 1>::THREADS,
-                                  (Layout<DIM, N, NSP, NS, FL == 1>::MINB > (FL == 1 ? DG_RHS_CAP1 : FL ? 6 : 5))
-                                      ? (FL == 1 ? DG_RHS_CAP1 : FL ? 6 : 5)
-                                      : Layout<DIM, N, NSP, NS, FL == 1>::MINB)
+__global__ void __launch_bounds__(Layout<DIM, N, NSP, NS, production_pair<FL>>::THREADS,
+                                  (Layout<DIM, N, NSP, NS, production_pair<FL>>::MINB > (production_pair<FL> ? DG_RHS_CAP1 : FL ? 6 : 5))
+                                      ? (production_pair<FL> ? DG_RHS_CAP1 : FL ? 6 : 5)
+                                      : Layout<DIM, N, NSP, NS, production_pair<FL>>::MINB)
 rhs_kernel(const DgArgs a, const KConst kc) {
   using S = Shape<DIM, N>;
-  using L = Layout<DIM, N, NSP, NS, FL == 1>;
+  using L = Layout<DIM, N, NSP, NS, production_pair<FL>>;
   constexpr int NV = L::NV, NP = L::NP, N1 = S::N1, EPB = L::EPB, NQ = L::NQ;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   real* sm = reinterpret_cast<real*>(smem_raw);
@@ -351,7 +355,7 @@ rhs_kernel(const DgArgs a, const KConst kc) {
   const int ne = (int)((a.K - e0) < EPB ? (a.K - e0) : EPB);
   const BasisTab<real>& B = c_tab[N];
   const bool read_du = a.mode == 1 && a.stage != 0;
-  const int vf = FL == 0 ? a.vf : FL == 1 ? (NSP == 1 ? DG_VF_RANOCHA : DG_VF_DUCROS) : FL - 2;
+  const int vf = FL == 0 ? a.vf : production_pair<FL> ? (NSP == 1 ? DG_VF_RANOCHA : DG_VF_DUCROS) : FL - 2;
   const int sf = FL ? DG_SF_LLF : a.sf;
   auto SW = [](int n) { return Swizzle<DIM, N>::at(n); };
 
@@ -671,7 +675,7 @@ rhs_kernel(const DgArgs a, const KConst kc) {
             fx[DIM] = bkind == DG_BC_ISOTHERMAL ? h : real(0);
           } else {  // inflow
             real r = 1;
-            if (FL < 2 && kc.suth_s > real(0))
+            if (FL <= 0 && kc.suth_s > real(0))
               r = sutherland_ratio(x.p * RealOps<real>::rcp(x.rho), kc.suth_s, kc.suth_c1, kc.suth_irt) *
                   RealOps<real>::rcp(sutherland_ratio(o.p * RealOps<real>::rcp(o.rho), kc.suth_s, kc.suth_c1,
                                                       kc.suth_irt));
@@ -908,7 +912,7 @@ rhs_kernel(const DgArgs a, const KConst kc) {
         }
         la *= ij;
         lv *= ij * ij * kc.visc * ir;
-        if (FL < 2 && kc.suth_s > real(0)) lv *= sutherland_ratio(p * ir, kc.suth_s, kc.suth_c1, kc.suth_irt);
+        if (FL <= 0 && kc.suth_s > real(0)) lv *= sutherland_ratio(p * ir, kc.suth_s, kc.suth_c1, kc.suth_irt);
         if (!(p > real(0)) || !isfinite(la)) {
           latch_status(a.status, DG_ST_NONPHYS, e0 + e);
           la = real(0);
@@ -1742,7 +1746,7 @@ cudaError_t set_smem(KernelT k, size_t bytes) {
 
 template <int DIM, int N, int NSP, bool NS, int FL, bool BND>
 cudaError_t launch_rhs_b(const DgArgs& a, cudaStream_t st) {
-  using L = Layout<DIM, N, NSP, NS, FL == 1>;
+  using L = Layout<DIM, N, NSP, NS, production_pair<FL>>;
   auto k = rhs_kernel<DIM, N, NSP, NS, FL, BND>;
   cudaError_t err = set_smem(k, L::SMEM);
   if (err != cudaSuccess) return err;
@@ -1755,7 +1759,7 @@ cudaError_t launch_rhs_b(const DgArgs& a, cudaStream_t st) {
 // compiled without boundary code (measured 5-7 % faster on the periodic Taylor-Green box)
 template <int DIM, int N, int NSP, bool NS, int FL = DG_FL>
 cudaError_t launch_rhs_t(const DgArgs& a, cudaStream_t st) {
-  if constexpr (FL == 1 && DIM == 3 && NSP == 1) {
+  if constexpr (production_pair<FL> && DIM == 3 && NSP == 1) {
     if (!a.has_bnd) return launch_rhs_b<DIM, N, NSP, NS, FL, false>(a, st);
   }
   return launch_rhs_b<DIM, N, NSP, NS, FL, true>(a, st);
@@ -1840,10 +1844,18 @@ cudaError_t DG_CAT(DG_PREFIX, _rhs)(const DgArgs& a, cudaStream_t st) {
     default: return cudaErrorInvalidValue;
   }
 }
+#elif defined(DG_SUTH_ONLY)
+// the production pair with Sutherland's law: one-gas Navier-Stokes in 3D
+#define DG_SUTH_CALL(DIM, N, NSP, X) DG_PREFIX::launch_rhs_t<DIM, N, NSP, true, -1>(a, st)
+cudaError_t DG_CAT(DG_PREFIX, _rhs)(const DgArgs& a, cudaStream_t st) {
+  if (a.dim == 3 && a.nsp == 1 && a.ns && a.suth_s > 0.0) { DG_DISPATCH_N(DG_SUTH_CALL, 3, 1, 0) }
+  return cudaErrorInvalidValue;
+}
 #else
 cudaError_t DG_CAT(DG_PREFIX, _rhs)(const DgArgs& a, cudaStream_t st) {
 #ifndef DG_GENERIC_ONLY
   const bool production = a.sf == DG_SF_LLF && a.vf == (a.nsp == 1 ? DG_VF_RANOCHA : DG_VF_DUCROS);
+  if (production && a.suth_s > 0.0) return DG_SUTH_RHS(a, st);
 #ifdef DG_SPLIT_RHS
   const bool split = a.dim == 3 && a.nsp == 1 && a.N == 3 && a.sf == DG_SF_LLF && !(a.suth_s > 0.0) &&
                      a.vf != DG_VF_RANOCHA;
@@ -1922,6 +1934,7 @@ cudaError_t DG_CAT(DG_PREFIX, _upload_basis)() {
   cudaError_t err = cudaMemcpyToSymbol(DG_PREFIX::c_tab, tab, sizeof(tab));
 #ifndef DG_GENERIC_ONLY
   if (err == cudaSuccess) err = DG_GENERIC_UPLOAD();
+  if (err == cudaSuccess) err = DG_SUTH_UPLOAD();
 #ifdef DG_SPLIT_UPLOAD
   if (err == cudaSuccess) err = DG_SPLIT_UPLOAD();
 #endif
