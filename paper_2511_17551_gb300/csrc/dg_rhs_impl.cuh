@@ -82,19 +82,36 @@ struct Swizzle {
   }
 };
 
-// resident-CTA target of the one-gas kernels: 8 (measured with the aliased layout below:
-// 9 and 10 CTAs of 96 threads cap the registers at 72 and 64, and the spills cost more than
-// the extra warps give back)
-#ifndef DG_RHS_CAP1
-#define DG_RHS_CAP1 8
-#endif
+// Shape of the right-hand-side CTAs: threads to fill with lines, and the resident CTAs the register
+// allocator is asked for.  What the registers of an SM allow goes by its four partitions (16,384
+// each): 18 warps leave one partition with 5 and cap all at 96 registers, 16 at 128.  Measured per
+// stage (mixed form unless said; smaller counts of CTAs leave the SM idle, larger ones spill):
+//   3D one gas, N = 3: 96 threads (2 elements), 8 CTAs; 9 and 10 cap the registers at 72 and 64
+//   3D one gas, N = 4: 160 threads (2 elements, 150 lines), 4 CTAs: 196 -> 162 us at 26^3 elements (96
+//     threads hold 75 lines, and at 8 CTAs spilled 128 bytes); Euler 134 -> 109, FP64 986 -> 831 (16^3)
+//   N = 7 without viscous terms: 2 CTAs, 161 -> 114 us (14^3; at 3 it spilled 548 bytes)
+//   2D: 128 threads (16 elements at N = 3), 7 CTAs, 96.3 -> 92.2 us (512 x 256)
+//   mixtures: 96 threads, 5 CTAs at N = 3 (131 -> 113 us, 28^3) and 4 at N = 4 (180 -> 171, 24^3) instead of
+//     192 threads and 3 CTAs; FP64 keeps 192 (300 against 337 us at 12^3)
+//   FP64 one gas: the FP64 pipe needs few warps, 4 CTAs (2D: 5) instead of 7 or 8 shed 700 to 1,700 bytes of
+//     spills: N = 3 Euler 1038 -> 996 us (24^3), N = 2 550 -> 521, 2D N = 3 529 -> 507
+template <int DIM, int N, int NSP>
+struct CtaShape {
+  static constexpr bool F64 = sizeof(real) == 8;
+  static constexpr int TPB = NSP > 1 ? (F64 ? 192 : 96) : DIM == 2 ? (F64 ? 96 : 128) : N == 4 ? 160 : 96;
+  static constexpr int CAP = NSP > 1  ? (F64 ? 3 : N == 3 ? 5 : 4)
+                             : F64      ? (DIM == 2 ? 5 : 4)
+                             : DIM == 2 ? 7
+                             : N == 4   ? 4
+                             : N == 7   ? 2
+                                        : 8;
+};
 template <int DIM, int N, int NSP, bool NS, bool AL = true>
 struct Layout {
   using S = Shape<DIM, N>;
   static constexpr int NV = NSP + DIM + 1;
   static constexpr int NP = S::NP;
-  // CTA shape (measured): one gas 96-thread CTAs, up to 8 per SM; mixtures 192 threads
-  static constexpr int EPB = epb<DIM, N, (NSP > 1 ? 192 : 96)>();
+  static constexpr int EPB = epb<DIM, N, CtaShape<DIM, N, NSP>::TPB>();
   static constexpr int NQ = DIM + 3;                // rho, v, p, beta(=rho/p)
   static constexpr int NFV = NS ? DIM * (DIM + 1) : 0;
   static constexpr int FACE_NODES = 2 * DIM * S::LPD;  // per element
@@ -130,10 +147,8 @@ struct Layout {
   static constexpr int FV = ACC + EPB * SACC;
   static constexpr int PC = FV + EPB * SFV;          // mixtures: p, c per node
   static constexpr int DU = PC + EPB * SPC;           // prefetched RK register du
-  // resident-CTA target (8 of the 96-thread CTAs for one gas; 3 for mixtures, whose
-  // 9-variable line accumulators spill below ~110 registers a thread), lowered where shared
-  // memory binds
-  static constexpr int CAP = NSP > 1 ? 3 : DG_RHS_CAP1;
+  // resident-CTA target, lowered where shared memory binds
+  static constexpr int CAP = CtaShape<DIM, N, NSP>::CAP;
   static constexpr int ctas_of(size_t bytes) {
     return (int)((227 * 1024) / (bytes + 1024)) >= CAP ? CAP : (int)((227 * 1024) / (bytes + 1024));
   }
@@ -321,17 +336,20 @@ __device__ __forceinline__ int outer_state(const DgArgs& a, const KConst& kc, in
 }
 
 // ------------------------------------------------------------------ main RHS / RK kernel
+// the runtime-choice kernel (FL = 0) carries more live branches: at most 5 CTAs per SM
+// (up to 136 registers a thread at 96 threads; 3 of the 160-thread CTAs of N = 4) instead of 8, so
+// that it does not spill; the split forms (FL >= 2) hold both nodes' conserved states per flux pair:
+// at most 6 (96 registers; at 7 the allocator is held to 80 and spills)
+template <int DIM, int N, int NSP, bool NS, int FL>
+constexpr int launch_ctas() {
+  constexpr int most = production_pair<FL> ? 8 : FL ? 6 : (DIM == 3 && N == 4 && NSP == 1) ? 3 : 5;
+  constexpr int minb = Layout<DIM, N, NSP, NS, production_pair<FL>>::MINB;
+  return minb > most ? most : minb;
+}
 // BND = false compiles the kernel for meshes without boundary faces (periodic or closed by
 // connectivity): the interface code then carries no boundary-state branches.
 template <int DIM, int N, int NSP, bool NS, int FL, bool BND = true>
-// the runtime-choice kernel (FL = 0) carries more live branches: at most 5 CTAs per SM
-// (up to 136 registers a thread at 96 threads) instead of 8, so that it does not spill;
-// the split forms (FL >= 2) hold both nodes' conserved states per flux pair: at most 6
-// (96 registers; at 7 the allocator is held to 80 and spills)
-__global__ void __launch_bounds__(Layout<DIM, N, NSP, NS, production_pair<FL>>::THREADS,
-                                  (Layout<DIM, N, NSP, NS, production_pair<FL>>::MINB > (production_pair<FL> ? DG_RHS_CAP1 : FL ? 6 : 5))
-                                      ? (production_pair<FL> ? DG_RHS_CAP1 : FL ? 6 : 5)
-                                      : Layout<DIM, N, NSP, NS, production_pair<FL>>::MINB)
+__global__ void __launch_bounds__(Layout<DIM, N, NSP, NS, production_pair<FL>>::THREADS, launch_ctas<DIM, N, NSP, NS, FL>())
 rhs_kernel(const DgArgs a, const KConst kc) {
   using S = Shape<DIM, N>;
   using L = Layout<DIM, N, NSP, NS, production_pair<FL>>;
