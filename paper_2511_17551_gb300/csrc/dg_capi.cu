@@ -511,6 +511,7 @@ DgArgs base_args(dg_ctx* c) {
   const bool f32 = c->precision == DG_MIXED;
   a.Ja = f32 ? (const void*)c->Ja32 : (const void*)c->Ja64;
   a.invJ = f32 ? (const void*)c->invJ32 : (const void*)c->invJ64;
+  a.own_metrics = 1;
   a.gradW = c->gradW;
   a.nbr = c->nbr;
   a.bc_kind = c->bc_kind;

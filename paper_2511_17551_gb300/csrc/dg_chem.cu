@@ -20,6 +20,7 @@
 #include "../../include/dg.h"
 #include "dg_dd.cuh"
 #include "dg_internal.h"
+#include "dg_launch.cuh"
 #include "dg_mlp.cuh"
 #include "dg_mlp_tc5.cuh"
 #include "dg_thermo.h"
@@ -381,6 +382,8 @@ chem_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, const doub
   typedef typename ChemForm<T>::type Form;
   __shared__ typename Form::Tab t;
   Form::stage(t, exp2);
+  pdl_wait();
+  if (sizeof(T) == 4) pdl_trigger();
   const int nv = NSPEC + dim + 1;
   typename ChemForm<T>::step dt;
   form_step(dtp ? *dtp : 0.0, dt);
@@ -974,15 +977,14 @@ cudaError_t dg_chem_source(DgThermo* th, const void* u, int f32, const double* d
   if (th->chem_mlp)
     return f32 ? chem_learned<float>(th, (const float*)u, dt_dev, refresh, s)
                : chem_learned<double>(th, (const double*)u, dt_dev, refresh, s);
+  const unsigned grid = grid_of(th->K * th->np);
+  const ChemTab32& tab = *(const ChemTab32*)th->chem_tab32;
+  const dgdd::dd* e2 = (const dgdd::dd*)th->chem_exp2;
   if (f32)
-    chem_kernel<float><<<grid_of(th->K * th->np), 128, 0, s>>>(
-        (const float*)u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr,
-        *(const ChemTab32*)th->chem_tab32, (const dgdd::dd*)th->chem_exp2, dt_dev, (float*)th->src);
-  else
-    chem_kernel<double><<<grid_of(th->K * th->np), 128, 0, s>>>(
-        (const double*)u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr,
-        *(const ChemTab32*)th->chem_tab32, (const dgdd::dd*)th->chem_exp2, dt_dev, (double*)th->src);
-  return cudaGetLastError();
+    return launch_pdl(chem_kernel<float>, grid, 128, 0, s, (const float*)u, th->T, th->K, th->np, th->dim, th->species_raw,
+                      th->reac, th->nr, tab, e2, dt_dev, (float*)th->src);
+  return launch_pdl(chem_kernel<double>, grid, 128, 0, s, (const double*)u, th->T, th->K, th->np, th->dim,
+                    th->species_raw, th->reac, th->nr, tab, e2, dt_dev, (double*)th->src);
 }
 
 cudaError_t dg_chem_mlp_set(DgThermo* th, const float* params_host, const double* st) {

@@ -18,6 +18,7 @@
 #pragma once
 #include <stdint.h>
 #include "dg_kernels.cuh"
+#include "dg_launch.cuh"
 
 #ifdef DG_GENERIC_ONLY
 #define DG_FL 0
@@ -29,6 +30,11 @@ namespace DG_PREFIX {
 
 using real = DG_REAL;
 using namespace dgk;
+
+// lets the next kernel's CTAs in (FP64: see dg_launch.cuh)
+__device__ __forceinline__ void trigger() {
+  if (sizeof(real) == 4) pdl_trigger();
+}
 
 // whether the kernel flavour FL fixes the production flux pair
 template <int FL>
@@ -414,11 +420,17 @@ rhs_kernel(const DgArgs a, const KConst kc) {
           bulk_g2s(dst + e * sstride, src + (e0 + e) * block, (unsigned)(RS * block), &s_bar);
         }
       };
+      // the context's metric terms are no kernel's output: requested before the preceding
+      // kernel has ended (a caller's own arrays may be)
+      if (!a.own_metrics) pdl_wait();
+      for (int j = tid; j < 2 * ne; j += 32) {
+        if (j & 1) copy(sja, L::SJA, (const real*)a.Ja, DIM * DIM * NP, j >> 1);
+        else copy(sij, L::SIJ, (const real*)a.invJ, NP, j >> 1);
+      }
+      pdl_wait();
       for (int j = tid; j < 8 * ne; j += 32) {
         const int e = j >> 3, kind = j & 7;
         if (kind == 0) copy(su, L::SU, (const real*)a.u, NV * NP, e);
-        if (kind == 1) copy(sja, L::SJA, (const real*)a.Ja, DIM * DIM * NP, e);
-        if (kind == 2) copy(sij, L::SIJ, (const real*)a.invJ, NP, e);
         if (kind == 3 && NSP > 1) copy(spc, L::SPC, (const real*)a.pc, 2 * NP, e);
         if (kind == 4 && NS) {
           if (L::FVD == DIM + 1) {
@@ -435,7 +447,9 @@ rhs_kernel(const DgArgs a, const KConst kc) {
           bulk_g2s(sacc + L::elo(e), (const real*)a.ulo + (e0 + e) * NV * NP + (NSP + DIM) * NP, RS * NP, &s_bar);
       }
     }
+    pdl_wait();
   } else {
+    pdl_wait();
     stage_strided<NV, L::SU, NP>(su, (const real*)a.u + e0 * NV * NP, ne, tid, nth);
     stage_strided<DIM * DIM, L::SJA, NP>(sja, (const real*)a.Ja + e0 * DIM * DIM * NP, ne, tid, nth);
     stage_strided<1, L::SIJ, NP>(sij, (const real*)a.invJ + e0 * NP, ne, tid, nth);
@@ -842,6 +856,7 @@ rhs_kernel(const DgArgs a, const KConst kc) {
     }
   }
   __syncthreads();
+  trigger();
 
   // ---- phase C: one thread per node and pass.
   real lam_a = 0, lam_v = 0;
@@ -956,6 +971,8 @@ rhs_kernel(const DgArgs a, const KConst kc) {
 // maxima in slot `slot`, or dt_fixed; adds the previous step's dt to the elapsed time
 // and clears the other slot for the coming step's reduction.
 __global__ void step_dt_kernel(const DgArgs a, int slot, int advance_time) {
+  pdl_wait();
+  trigger();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   if (advance_time) a.scal[0] += a.scal[1];
   double dt = a.dt_fixed;
@@ -1234,6 +1251,8 @@ __global__ void __launch_bounds__(128) positivity_kernel(const DgArgs a, real* u
   constexpr int NP = S::NP, NV = NSP + DIM + 1;
   constexpr int EPW = NP >= 128 ? 1 : 128 / NP;
   static_assert(EPW <= 32, "flag mask");
+  pdl_wait();
+  trigger();
   const int lane = threadIdx.x & 31;
   const int64_t k0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * EPW;
   if (k0 >= a.K) return;  // uniform per warp
@@ -1338,13 +1357,17 @@ gradient_kernel(const DgArgs a, const KConst kc) {
     if (tid == 0) {
       mbar_init(&s_bar);
       mbar_expect(&s_bar, (unsigned)(RS * NP * ne * (DIM * DIM + 1 + NV)));
+      if (!a.own_metrics) pdl_wait();
       bulk_g2s(sja, (const real*)a.Ja + e0 * DIM * DIM * NP, RS * ne * DIM * DIM * NP, &s_bar);
       bulk_g2s(sij, (const real*)a.invJ + e0 * NP, RS * ne * NP, &s_bar);
+      pdl_wait();
       bulk_g2s(sg, gu + e0 * NV * NP, RS * ne * NV * NP, &s_bar);
     }
+    pdl_wait();
     __syncthreads();  // the barrier is initialised before anyone polls it
     if (!mbar_wait0(&s_bar)) latch_status(a.status, DG_ST_TIMEOUT, e0);
   } else {
+    pdl_wait();
     stage_async(sja, (const real*)a.Ja + e0 * DIM * DIM * NP, ne * DIM * DIM * NP, tid, nth);
     stage_async(sij, (const real*)a.invJ + e0 * NP, ne * NP, tid, nth);
     stage_async(sg, gu + e0 * NV * NP, ne * NV * NP, tid, nth);
@@ -1436,6 +1459,7 @@ gradient_kernel(const DgArgs a, const KConst kc) {
       for (int c = 0; c < NW; ++c) g[c * NP + SWZ(base + i * s)] = G[i][c];
   }
   __syncthreads();
+  trigger();
   // physical gradients G_x = (1/J) sum_d Ja^d_x Q_d; written as they are (grad_mode 1) or
   // turned into the contravariant viscous fluxes sum_x Ja^d_x f^v_x(G; v, mu(T)) that the
   // right-hand-side kernel consumes (grad_mode 0)
@@ -1496,6 +1520,8 @@ template <int DIM, int N, int NSP>
 __global__ void boundary_lift_kernel(const DgArgs a, const KConst kc) {
   using S = Shape<DIM, N>;
   constexpr int NV = NSP + DIM + 1, NP = S::NP, N1 = S::N1, NW = DIM + 1;
+  pdl_wait();
+  trigger();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= a.K * NP) return;
   const int64_t e = i / NP;
@@ -1592,6 +1618,8 @@ template <int DIM, int NSP>
 __global__ void lambda_kernel(const DgArgs a, const KConst kc, int slot) {
   __shared__ unsigned long long s_l[2];
   constexpr int NV = NSP + DIM + 1;
+  pdl_wait();
+  trigger();
   const int np = a.np;
   const int64_t n = a.K * np;
   if (threadIdx.x == 0) s_l[0] = s_l[1] = 0ull;
@@ -1681,6 +1709,8 @@ __global__ void __launch_bounds__(IndShape<DIM, N>::THREADS) indicator_kernel(co
   using I = IndShape<DIM, N>;
   constexpr int NP = S::NP, N1 = S::N1, NV = NSP + DIM + 1, ROW = I::ROW;
   __shared__ real sf[I::EPC * ROW];
+  pdl_wait();
+  trigger();
   const BasisTab<real>& B = c_tab[N];
   const int tid = threadIdx.x;
   const int64_t e0 = (int64_t)blockIdx.x * I::EPC;
@@ -1769,8 +1799,7 @@ cudaError_t launch_rhs_b(const DgArgs& a, cudaStream_t st) {
   cudaError_t err = set_smem(k, L::SMEM);
   if (err != cudaSuccess) return err;
   const int64_t grid = (a.K + L::EPB - 1) / L::EPB;
-  k<<<(unsigned)grid, L::THREADS, L::SMEM, st>>>(a, make_kconst(a));
-  return cudaGetLastError();
+  return launch_pdl(k, (unsigned)grid, L::THREADS, L::SMEM, st, a, make_kconst(a));
 }
 
 // the production pair of a one-gas 3D mesh without boundary faces runs the kernel
@@ -1792,12 +1821,10 @@ cudaError_t launch_grad_t(const DgArgs& a, cudaStream_t st) {
   cudaError_t err = set_smem(k, smem);
   if (err != cudaSuccess) return err;
   const int64_t grid = (a.K + L::EPB - 1) / L::EPB;
-  k<<<(unsigned)grid, L::THREADS, smem, st>>>(a, make_kconst(a));
-  err = cudaGetLastError();
+  err = launch_pdl(k, (unsigned)grid, L::THREADS, smem, st, a, make_kconst(a));
   if (err != cudaSuccess || !a.has_bnd) return err;
   const int64_t nn = a.K * Shape<DIM, N>::NP;
-  boundary_lift_kernel<DIM, N, NSP><<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(a, make_kconst(a));
-  return cudaGetLastError();
+  return launch_pdl(boundary_lift_kernel<DIM, N, NSP>, (unsigned)((nn + 255) / 256), 256, 0, st, a, make_kconst(a));
 }
 
 template <int DIM, int N, int NSP>
@@ -1806,16 +1833,15 @@ cudaError_t launch_pos_t(const DgArgs& a, void* u, void* ulo, double eps, unsign
   constexpr int NP = Shape<DIM, N>::NP, EPW = NP >= 128 ? 1 : 128 / NP;
   const int64_t warps = (a.K + EPW - 1) / EPW;
   const int64_t grid = (warps * 32 + 127) / 128;
-  positivity_kernel<DIM, N, NSP><<<(unsigned)grid, 128, 0, st>>>(a, (real*)u, (real*)ulo, eps, nlim);
-  return cudaGetLastError();
+  return launch_pdl(positivity_kernel<DIM, N, NSP>, (unsigned)grid, 128, 0, st, a, (real*)u, (real*)ulo, eps, nlim);
 }
 
 template <int DIM, int N, int NSP>
 cudaError_t launch_ind_t(const DgArgs& a, double amax, void* out, cudaStream_t st) {
   using I = IndShape<DIM, N>;
   const int64_t grid = (a.K + I::EPC - 1) / I::EPC;
-  indicator_kernel<DIM, N, NSP><<<(unsigned)grid, I::THREADS, 0, st>>>(a, make_kconst(a), (real)amax, (real*)out);
-  return cudaGetLastError();
+  return launch_pdl(indicator_kernel<DIM, N, NSP>, (unsigned)grid, I::THREADS, 0, st, a, make_kconst(a), (real)amax,
+                    (real*)out);
 }
 #endif  // DG_GENERIC_ONLY
 
@@ -1916,16 +1942,17 @@ cudaError_t DG_CAT(DG_PREFIX, _lambda)(const DgArgs& a, int slot, cudaStream_t s
   int64_t grid = (n + bs - 1) / bs;
   if (grid > 152 * 16) grid = 152 * 16;
   const DG_PREFIX::KConst kc = DG_PREFIX::make_kconst(a);
-  if (a.dim == 3 && a.nsp == 1) DG_PREFIX::lambda_kernel<3, 1><<<(unsigned)grid, bs, 0, st>>>(a, kc, slot);
-  else if (a.dim == 2 && a.nsp == 1) DG_PREFIX::lambda_kernel<2, 1><<<(unsigned)grid, bs, 0, st>>>(a, kc, slot);
-  else if (a.dim == 3 && a.nsp == 5) DG_PREFIX::lambda_kernel<3, 5><<<(unsigned)grid, bs, 0, st>>>(a, kc, slot);
-  else return cudaErrorInvalidValue;
-  return cudaGetLastError();
+  if (a.dim == 3 && a.nsp == 1)
+    return launch_pdl(DG_PREFIX::lambda_kernel<3, 1>, (unsigned)grid, bs, 0, st, a, kc, slot);
+  if (a.dim == 2 && a.nsp == 1)
+    return launch_pdl(DG_PREFIX::lambda_kernel<2, 1>, (unsigned)grid, bs, 0, st, a, kc, slot);
+  if (a.dim == 3 && a.nsp == 5)
+    return launch_pdl(DG_PREFIX::lambda_kernel<3, 5>, (unsigned)grid, bs, 0, st, a, kc, slot);
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t DG_CAT(DG_PREFIX, _step_dt)(const DgArgs& a, int slot, int advance_time, cudaStream_t st) {
-  DG_PREFIX::step_dt_kernel<<<1, 32, 0, st>>>(a, slot, advance_time);
-  return cudaGetLastError();
+  return launch_pdl(DG_PREFIX::step_dt_kernel, 1, 32, 0, st, a, slot, advance_time);
 }
 
 #endif  // DG_GENERIC_ONLY

@@ -21,6 +21,7 @@
 
 #include "dg_dd.cuh"
 #include "dg_internal.h"
+#include "dg_launch.cuh"
 #include "dg_thermo.h"
 
 #define DG_RU 8.314462618
@@ -77,6 +78,7 @@ __device__ __forceinline__ bool newton64(const Poly<double>& P, double e, double
 // FP64 form: the full FP64 Newton iteration, one thread per node
 __global__ void thermo_update_kernel(const double* u, int64_t K, int np, int dim, const double* cf, double* Tc,
                                      double* pc, unsigned long long* status) {
+  pdl_wait();
   const int nv = NSPEC + dim + 1;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < K * np;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -147,6 +149,8 @@ __global__ void __launch_bounds__(256, 3) thermo_mixed_kernel(const float* u, in
   __shared__ dd b0s[NSPEC];
   if (threadIdx.x < 8 * NSPEC) c32[threadIdx.x] = cf32[threadIdx.x];
   if (threadIdx.x < NSPEC) b0s[threadIdx.x] = from_double(cf[8 * threadIdx.x]);
+  pdl_wait();
+  pdl_trigger();
   __syncthreads();
   for (int64_t base = blockIdx.x * (int64_t)256; base < K * NP; base += gridDim.x * (int64_t)256) {
     // element and node of base + threadIdx.x: the 64-bit division is the same in all threads
@@ -346,19 +350,17 @@ cudaError_t dg_thermo_reset(DgThermo* th, cudaStream_t s) {
 
 cudaError_t dg_thermo_update(DgThermo* th, const void* u, int f32, cudaStream_t s) {
   if (th->mode == 1 && th->mlp) return dg_mlp_thermo_update(th, u, f32, s);
-  if (!f32) {
-    thermo_update_kernel<<<grid_of(th->K * th->np), 256, 0, s>>>((const double*)u, th->K, th->np, th->dim, th->species,
-                                                                 th->T, (double*)th->pc, th->status);
-  } else if (th->dim == 3 && th->np == 64) {
-    thermo_mixed_kernel<64, 3><<<grid_of(th->K * th->np), 256, 0, s>>>((const float*)u, th->K, th->species, th->coef32,
-                                                                       th->T, (float*)th->pc, th->status);
-  } else if (th->dim == 3 && th->np == 125) {
-    thermo_mixed_kernel<125, 3><<<grid_of(th->K * th->np), 256, 0, s>>>((const float*)u, th->K, th->species, th->coef32,
-                                                                        th->T, (float*)th->pc, th->status);
-  } else {
-    return cudaErrorInvalidValue;  // mixtures are 3D with N = 3 or 4
-  }
-  return cudaGetLastError();
+  const unsigned grid = grid_of(th->K * th->np);
+  if (!f32)
+    return launch_pdl(thermo_update_kernel, grid, 256, 0, s, (const double*)u, th->K, th->np, th->dim, th->species, th->T,
+                      (double*)th->pc, th->status);
+  if (th->dim == 3 && th->np == 64)
+    return launch_pdl(thermo_mixed_kernel<64, 3>, grid, 256, 0, s, (const float*)u, th->K, th->species, th->coef32, th->T,
+                      (float*)th->pc, th->status);
+  if (th->dim == 3 && th->np == 125)
+    return launch_pdl(thermo_mixed_kernel<125, 3>, grid, 256, 0, s, (const float*)u, th->K, th->species, th->coef32, th->T,
+                      (float*)th->pc, th->status);
+  return cudaErrorInvalidValue;  // mixtures are 3D with N = 3 or 4
 }
 
 cudaError_t dg_thermo_boundary(DgThermo* th, const double* bw, int n_bc, void* bc_u, cudaStream_t s) {
