@@ -41,12 +41,36 @@ struct BasisTab {
 };
 
 template <typename real> struct RealOps;
+// FP64 reciprocal and square root from the hardware's approximations (rcp.approx.ftz.f64 and
+// rsqrt.approx.ftz.f64: relative error about 2^-22) and one cubically convergent step each: with
+// e = 1 - x y the reciprocal is y (1 + e + e^2 + ...), with e = 1 - x y^2 the square root is
+// x y (1 + e/2 + 3 e^2/8 + ...) (Householder's method of order three); what is cut off is below
+// 2^-63.  3 and 5 operations of the FP64 pipe, which bounds the FP64 kernels.  Zeros, infinities
+// and NaN give what they should by integer tests and selects (a branch to the general functions for
+// them cost more than the operations saved); subnormal arguments count as zeros, subnormal
+// reciprocals are zeros.  FP64 right-hand side of the 32^3 N = 3 Navier-Stokes mesh with __drcp_rn
+// and sqrt 2534 us, with these 2372 us.
 template <> struct RealOps<double> {
-  static __device__ __forceinline__ double rcp(double x) { return __drcp_rn(x); }
-  static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
+  static __device__ __forceinline__ double rcp(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    const double r = fma(fma(e, e, e), y, y);
+    return ((unsigned)__double2hiint(e) & 0x7fffffffu) < 0x3ff00000u ? r : y;  // |e| < 1, not NaN
+  }
+  static __device__ __forceinline__ double sqrt_(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double t = x * y;
+    const double e = fma(-t, y, 1.0);
+    const double r = fma(t * e, fma(e, 0.375, 0.5), t);
+    const unsigned h = (unsigned)__double2hiint(x);
+    return (h & 0x7ff00000u) == 0u || h == 0x7ff00000u ? x : r;
+  }
+  // 0 <= f2 < about 1e-4 (the high word decides; false for NaN)
+  static __device__ __forceinline__ bool near(double f2) { return (unsigned)__double2hiint(f2) < 0x3f1a36e2u; }
   static __device__ __forceinline__ double log_(double x) { return log(x); }
   static __device__ __forceinline__ double div(double a, double b) { return a / b; }
-  static constexpr double ln_eps = 1e-4;
 };
 template <> struct RealOps<float> {
   // single MUFU reciprocal / reciprocal square root (<= 2 ulp): the mixed form's
@@ -56,7 +80,7 @@ template <> struct RealOps<float> {
   static __device__ __forceinline__ float log_(float x) { return logf(x); }
   static __device__ __forceinline__ float div(float a, float b) { return __fdiv_rn(a, b); }
   // the artanh series truncated after f^6 has relative error f^8/9: 1.1e-9 at 1e-2
-  static constexpr float ln_eps = 1e-2f;
+  static __device__ __forceinline__ bool near(float f2) { return f2 < 1e-2f; }
 };
 
 // logarithmic mean L(x,y) = (y-x)/ln(y/x): artanh series for nearly equal
@@ -66,12 +90,13 @@ __device__ __forceinline__ real ln_mean(real x, real y) {
   real s = x + y, d = y - x;
   real rs = RealOps<real>::rcp(s);
   real f = d * rs, f2 = f * f;
-  if (f2 < RealOps<real>::ln_eps) {
+  if (RealOps<real>::near(f2)) {
     if (sizeof(real) == 8) {
-      // L = (s/2) / (1 + x), x = f2 (1/3 + f2 (1/5 + f2/7)) <= 3.4e-5: the geometric series
-      // to x^3 is exact to FP64 rounding (x^4 < 2e-18) and needs no second reciprocal
-      const real x = f2 * (real(1.0 / 3.0) + f2 * (real(1.0 / 5.0) + f2 * real(1.0 / 7.0)));
-      return real(0.5) * s * (real(1) - x * (real(1) - x * (real(1) - x)));
+      // L = (s/2) f / artanh(f), f / artanh(f) = 1 - f2/3 - 4 f2^2/45 - 44 f2^3/945 - ...: the
+      // next term is below 3.1e-18, and there is no second reciprocal
+      const real x = f2 * (real(1.0 / 3.0) + f2 * (real(4.0 / 45.0) + f2 * real(44.0 / 945.0)));
+      const real h = real(0.5) * s;
+      return h - h * x;
     }
     real poly = real(2) + f2 * (real(2.0 / 3.0) + f2 * (real(2.0 / 5.0) + f2 * real(2.0 / 7.0)));
     return s * RealOps<real>::rcp(poly);
@@ -85,7 +110,7 @@ __device__ __forceinline__ real inv_ln_mean(real x, real y) {
   real s = x + y, d = y - x;
   real rs = RealOps<real>::rcp(s);
   real f = d * rs, f2 = f * f;
-  if (f2 < RealOps<real>::ln_eps) {
+  if (RealOps<real>::near(f2)) {
     real poly = real(2) + f2 * (real(2.0 / 3.0) + f2 * (real(2.0 / 5.0) + f2 * real(2.0 / 7.0)));
     return poly * rs;
   }
@@ -102,7 +127,7 @@ __device__ __forceinline__ void ln_mean_pair(float xr, float yr, float xb, float
   const float2 rs = make_float2(RealOps<float>::rcp(s.x), RealOps<float>::rcp(s.y));
   const float2 f = __fmul2_rn(d, rs);
   const float2 f2 = __fmul2_rn(f, f);
-  if (f2.x < RealOps<float>::ln_eps && f2.y < RealOps<float>::ln_eps) {
+  if (RealOps<float>::near(f2.x) && RealOps<float>::near(f2.y)) {
     float2 poly = __ffma2_rn(f2, make_float2(2.f / 7.f, 2.f / 7.f), make_float2(2.f / 5.f, 2.f / 5.f));
     poly = __ffma2_rn(f2, poly, make_float2(2.f / 3.f, 2.f / 3.f));
     poly = __ffma2_rn(f2, poly, make_float2(2.f, 2.f));
@@ -149,6 +174,7 @@ struct NodeState {
   static constexpr int NV = NSP + DIM + 1;
   real u[NV];
   real rho, v[DIM], p, c, pp;
+  real cc;  // c^2 (one gas)
 };
 
 // pref, eref = pref / (gamma - 1): pressure offset; elo: low part of the compensated
@@ -170,15 +196,25 @@ __device__ __forceinline__ bool prim_from_cons(NodeState<real, DIM, NSP>& s, rea
     ke += s.u[NSP + d] * s.v[d];
   }
   if (NSP == 1) {
-    s.pp = (gamma - real(1)) * (((s.u[NSP + DIM] - eref) + elo) - real(0.5) * ke);
+    const real de = sizeof(real) == 4 ? (s.u[NSP + DIM] - eref) + elo : s.u[NSP + DIM] - eref;  // elo: FP32 only
+    s.pp = (gamma - real(1)) * (de - real(0.5) * ke);
     s.p = s.pp + pref;
-    s.c = RealOps<real>::sqrt_(gamma * s.p * ir);
+    s.cc = gamma * s.p * ir;
+    s.c = RealOps<real>::sqrt_(s.cc);
   } else {
     s.p = p_ext;
     s.pp = p_ext - pref;
     s.c = c_ext;
   }
   return rho > real(0) && s.p > real(0) && isfinite(s.p);
+}
+
+// c |n| from nn = |n|^2: in FP64 one square root of the product (its range is no concern there),
+// the norm's own being left out; in FP32 the product of the two
+template <typename real, int DIM, int NSP>
+__device__ __forceinline__ real acoustic(const NodeState<real, DIM, NSP>& s, real nn) {
+  if (sizeof(real) == 8 && NSP == 1) return RealOps<real>::sqrt_(s.cc * nn);
+  return s.c * RealOps<real>::sqrt_(nn);
 }
 
 template <typename real, int DIM, int NSP>
@@ -200,7 +236,8 @@ __device__ __forceinline__ void surface_flux(int sf, const NodeState<real, DIM, 
                                              const NodeState<real, DIM, NSP>& R, const real* n,
                                              real inv_gm1, real pref, real* f);
 
-// two-point volume flux F#(L, R; n); pL, pR are shifted pressures p - pref (momentum
+// twice the two-point volume flux F#(L, R; n) (every mean is left a sum; the caller's coefficient
+// takes the half: a power of two, so the result is the same to the bit); pL, pR are shifted pressures p - pref (momentum
 // components), bL, bR = rho / p of the full pressures
 template <typename real, int DIM, int NSP>
 __device__ __forceinline__ void volume_flux(int vf, real rL, const real* vL, real pL, real bL,
@@ -233,22 +270,24 @@ __device__ __forceinline__ void volume_flux(int vf, real rL, const real* vL, rea
     real vv = 0;
 #pragma unroll
     for (int d = 0; d < DIM; ++d) vv += vL[d] * vR[d];
-    real frho = rho_m * real(0.5) * (vnL + vnR);
-    real pa = real(0.5) * (pL + pR);
+    const real sn = vnL + vnR;
+    real frho = rho_m * sn;
+    const real hrho = real(0.5) * frho;
+    real pa = pL + pR;
     f[0] = frho;
 #pragma unroll
-    for (int d = 0; d < DIM; ++d) f[1 + d] = frho * real(0.5) * (vL[d] + vR[d]) + pa * n[d];
-    f[1 + DIM] = frho * (real(0.5) * vv + ib * inv_gm1) + real(0.5) * ((pL + pref) * vnR + (pR + pref) * vnL);
+    for (int d = 0; d < DIM; ++d) f[1 + d] = hrho * (vL[d] + vR[d]) + pa * n[d];
+    f[1 + DIM] = frho * (real(0.5) * vv + ib * inv_gm1) + (pL * vnR + pR * vnL + pref * sn);
   } else if (NSP == 1 && (vf == DG_VF_KG || vf == DG_VF_PIROZZOLI)) {
     // Kennedy-Gruber / Pirozzoli split forms as products of arithmetic means
-    const real frho = real(0.25) * (rL + rR) * (vnL + vnR);
+    const real frho = real(0.5) * (rL + rR) * (vnL + vnR);
     const real irL = RealOps<real>::rcp(rL), irR = RealOps<real>::rcp(rR);
     f[0] = frho;
 #pragma unroll
-    for (int d = 0; d < DIM; ++d) f[1 + d] = frho * real(0.5) * (vL[d] + vR[d]) + real(0.5) * (pL + pR) * n[d];
+    for (int d = 0; d < DIM; ++d) f[1 + d] = frho * real(0.5) * (vL[d] + vR[d]) + (pL + pR) * n[d];
     if (vf == DG_VF_KG)
       f[1 + DIM] = frho * real(0.5) * (uL[1 + DIM] * irL + uR[1 + DIM] * irR) +
-                   real(0.25) * ((pL + pref) + (pR + pref)) * (vnL + vnR);
+                   real(0.5) * ((pL + pref) + (pR + pref)) * (vnL + vnR);
     else
       f[1 + DIM] = frho * real(0.5) * ((uL[1 + DIM] + (pL + pref)) * irL + (uR[1 + DIM] + (pR + pref)) * irR);
   } else if (NSP == 1 && vf == DG_VF_MORINISHI) {
@@ -260,33 +299,32 @@ __device__ __forceinline__ void volume_flux(int vf, real rL, const real* vL, rea
       frho += (uL[1 + d] + uR[1 + d]) * n[d];
       vv += vL[d] * vR[d];
     }
-    frho *= real(0.5);
     f[0] = frho;
 #pragma unroll
-    for (int d = 0; d < DIM; ++d) f[1 + d] = frho * real(0.5) * (vL[d] + vR[d]) + real(0.5) * (pL + pR) * n[d];
-    f[1 + DIM] = (real(1) + inv_gm1) * real(0.5) * ((pL + pref) * vnL + (pR + pref) * vnR) + frho * real(0.5) * vv;
+    for (int d = 0; d < DIM; ++d) f[1 + d] = frho * real(0.5) * (vL[d] + vR[d]) + (pL + pR) * n[d];
+    f[1 + DIM] = (real(1) + inv_gm1) * ((pL + pref) * vnL + (pR + pref) * vnR) + frho * real(0.5) * vv;
   } else if (vf == DG_VF_DUCROS) {
     real vn = real(0.5) * (vnL + vnR);
-    real pa = real(0.5) * (pL + pR);
+    real pa = pL + pR;
 #pragma unroll
-    for (int k = 0; k < NSP; ++k) f[k] = real(0.5) * (uL[k] + uR[k]) * vn;
+    for (int k = 0; k < NSP; ++k) f[k] = (uL[k] + uR[k]) * vn;
 #pragma unroll
-    for (int d = 0; d < DIM; ++d) f[NSP + d] = real(0.5) * (uL[NSP + d] + uR[NSP + d]) * vn + pa * n[d];
-    f[NSP + DIM] = real(0.5) * (uL[NSP + DIM] + (pL + pref) + uR[NSP + DIM] + (pR + pref)) * vn;
+    for (int d = 0; d < DIM; ++d) f[NSP + d] = (uL[NSP + d] + uR[NSP + d]) * vn + pa * n[d];
+    f[NSP + DIM] = (uL[NSP + DIM] + (pL + pref) + uR[NSP + DIM] + (pR + pref)) * vn;
   } else {  // central
 #pragma unroll
-    for (int k = 0; k < NSP; ++k) f[k] = real(0.5) * (uL[k] * vnL + uR[k] * vnR);
+    for (int k = 0; k < NSP; ++k) f[k] = uL[k] * vnL + uR[k] * vnR;
 #pragma unroll
     for (int d = 0; d < DIM; ++d)
-      f[NSP + d] = real(0.5) * (uL[NSP + d] * vnL + pL * n[d] + uR[NSP + d] * vnR + pR * n[d]);
-    f[NSP + DIM] = real(0.5) * ((uL[NSP + DIM] + (pL + pref)) * vnL + (uR[NSP + DIM] + (pR + pref)) * vnR);
+      f[NSP + d] = uL[NSP + d] * vnL + pL * n[d] + uR[NSP + d] * vnR + pR * n[d];
+    f[NSP + DIM] = (uL[NSP + DIM] + (pL + pref)) * vnL + (uR[NSP + DIM] + (pR + pref)) * vnR;
   }
   (void)NV;
 }
 
-// LLF flux between the own state o and the other side's state x for either orientation
+// twice the LLF flux between the own state o and the other side's state x for either orientation
 // with one code instance: F(L, R) with (L, R) = (o, x) when own_left, (x, o) otherwise;
-// bit for bit the same as surface_flux(DG_SF_LLF, L, R, ...) (the mean and the maximum
+// bit for bit twice surface_flux(DG_SF_LLF, L, R, ...) (the sum and the maximum
 // are symmetric, the jump only changes sign)
 template <typename real, int DIM, int NSP>
 __device__ __forceinline__ void llf_oriented(const NodeState<real, DIM, NSP>& o, const NodeState<real, DIM, NSP>& x,
@@ -299,14 +337,13 @@ __device__ __forceinline__ void llf_oriented(const NodeState<real, DIM, NSP>& o,
     vno += o.v[d] * n[d];
     vnx += x.v[d] * n[d];
   }
-  nn = RealOps<real>::sqrt_(nn);
   real fo[NV], fx[NV];
   phys_flux<real, DIM, NSP>(o, n, fo);
   phys_flux<real, DIM, NSP>(x, n, fx);
-  const real lam = fmax(fabs(vno) + o.c * nn, fabs(vnx) + x.c * nn);
-  const real hl = own_left ? real(0.5) * lam : real(-0.5) * lam;
+  const real lam = fmax(fabs(vno) + acoustic<real, DIM, NSP>(o, nn), fabs(vnx) + acoustic<real, DIM, NSP>(x, nn));
+  const real hl = own_left ? lam : -lam;
 #pragma unroll
-  for (int k = 0; k < NV; ++k) f[k] = real(0.5) * (fo[k] + fx[k]) - hl * (x.u[k] - o.u[k]);
+  for (int k = 0; k < NV; ++k) f[k] = (fo[k] + fx[k]) - hl * (x.u[k] - o.u[k]);
 }
 
 template <typename real, int DIM, int NSP>
@@ -318,6 +355,8 @@ __device__ __forceinline__ void surface_flux(int sf, const NodeState<real, DIM, 
     real bL = L.rho * RealOps<real>::rcp(L.p), bR = R.rho * RealOps<real>::rcp(R.p);
     volume_flux<real, DIM, NSP>(NSP == 1 ? DG_VF_RANOCHA : DG_VF_DUCROS, L.rho, L.v, L.pp, bL, L.u,
                                 R.rho, R.v, R.pp, bR, R.u, n, inv_gm1, pref, f);
+#pragma unroll
+    for (int k = 0; k < NV; ++k) f[k] *= real(0.5);
     return;
   }
   real nn = 0, vnL = 0, vnR = 0;
@@ -327,17 +366,17 @@ __device__ __forceinline__ void surface_flux(int sf, const NodeState<real, DIM, 
     vnL += L.v[d] * n[d];
     vnR += R.v[d] * n[d];
   }
-  nn = RealOps<real>::sqrt_(nn);
   real fL[NV], fR[NV];
   phys_flux<real, DIM, NSP>(L, n, fL);
   phys_flux<real, DIM, NSP>(R, n, fR);
   if (sf == DG_SF_LLF) {
-    real lam = fmax(fabs(vnL) + L.c * nn, fabs(vnR) + R.c * nn);
+    real lam = fmax(fabs(vnL) + acoustic<real, DIM, NSP>(L, nn), fabs(vnR) + acoustic<real, DIM, NSP>(R, nn));
 #pragma unroll
     for (int k = 0; k < NV; ++k) f[k] = real(0.5) * (fL[k] + fR[k]) - real(0.5) * lam * (R.u[k] - L.u[k]);
     return;
   }
   // HLLC along n/|n| with Davis speed estimates, scaled by |n|
+  nn = RealOps<real>::sqrt_(nn);
   real inn = RealOps<real>::rcp(nn);
   real uLn = vnL * inn, uRn = vnR * inn;
   real SL = fmin(uLn - L.c, uRn - R.c);

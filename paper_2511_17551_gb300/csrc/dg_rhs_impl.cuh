@@ -566,8 +566,9 @@ rhs_kernel(const DgArgs a, const KConst kc) {
       }
       real p, pp;
       if (NSP == 1) {
-        const real elo = have_elo ? sacc[L::elo(e) + n] : real(0);
-        pp = kc.gm1 * (((uu[(NSP + DIM) * NP] - kc.eref) + elo) - real(0.5) * ke);
+        real de = uu[(NSP + DIM) * NP] - kc.eref;
+        if (sizeof(real) == 4) de += have_elo ? sacc[L::elo(e) + n] : real(0);
+        pp = kc.gm1 * (de - real(0.5) * ke);
         p = pp + kc.pref;
       } else {
         pcv[0] = spc[e * L::SPC + n];
@@ -665,8 +666,12 @@ rhs_kernel(const DgArgs a, const KConst kc) {
       for (int c = 0; c < DIM; ++c) o.v[c] = q[(1 + c) * NP + node];
       o.pp = q[(1 + DIM) * NP + node];
       o.p = o.pp + kc.pref;
-      o.c = NSP == 1 ? RealOps<real>::sqrt_(kc.gamma * o.p * RealOps<real>::rcp(o.rho))
-                     : spc[e * L::SPC + NP + node];
+      if (NSP == 1) {
+        o.cc = kc.gamma * o.p * RealOps<real>::rcp(o.rho);
+        o.c = RealOps<real>::sqrt_(o.cc);
+      } else {
+        o.c = spc[e * L::SPC + NP + node];
+      }
       real nface[DIM];
 #pragma unroll
       for (int c = 0; c < DIM; ++c) nface[c] = ja[c * NP + node];
@@ -684,6 +689,9 @@ rhs_kernel(const DgArgs a, const KConst kc) {
 #pragma unroll
       for (int c = 0; c <= DIM; ++c) vl[c] = 0;
       const bool visc = NS && bkind != DG_BC_OUTFLOW;
+      // weight of the jump to the other side's flux, of which the mean takes half (in FP32 the half
+      // goes to the jump itself: a value less to keep)
+      real wv = sizeof(real) == 4 ? iw : real(0.5) * iw;
       if (visc) {
         // viscous interface flux: mean of both sides' f^v . n, lifted as (Fv* - Fv).  At a
         // boundary the other side follows from the own flux (the flux is linear in the
@@ -721,19 +729,25 @@ rhs_kernel(const DgArgs a, const KConst kc) {
           }
         }
 #pragma unroll
-        for (int c = 0; c <= DIM; ++c) vl[c] = wall ? fx[c] - fvd[c * NP] : real(0.5) * (fx[c] - fvd[c * NP]);
+        for (int c = 0; c <= DIM; ++c) {
+          vl[c] = fx[c] - fvd[c * NP];
+          if (sizeof(real) == 4 && !wall) vl[c] *= real(0.5);
+        }
+        if (wall) wv = iw;
       }
-      // the end node's sums take the lifted terms: + iw F*, then - iw (Fv* - Fv)
+      // the end node's sums take the lifted terms: + iw F* (llf_oriented gives twice F*), then
+      // - iw (Fv* - Fv)
+      const real wf = (FL && !phys) ? real(0.5) * iw : iw;
 #pragma unroll
       for (int k = 0; k < NV; ++k) {
-        if (side) acc[N][k] += iw * Fs[k];
-        else acc[0][k] += iw * Fs[k];
+        if (side) acc[N][k] += wf * Fs[k];
+        else acc[0][k] += wf * Fs[k];
       }
       if (visc) {
 #pragma unroll
         for (int c = 0; c <= DIM; ++c) {
-          if (side) acc[N][NSP + c] -= iw * vl[c];
-          else acc[0][NSP + c] -= iw * vl[c];
+          if (side) acc[N][NSP + c] -= wv * vl[c];
+          else acc[0][NSP + c] -= wv * vl[c];
         }
       }
     }
@@ -741,9 +755,9 @@ rhs_kernel(const DgArgs a, const KConst kc) {
     const real al = s_alpha[e];
     const real wdg = real(1) - al;
     // every two-point flux is linear in the normal: F(n_i + n_l) = 2 F((n_i + n_l) / 2)
-    // exactly (a power-of-two scale), so the pair's mean normal is left unhalved and the
-    // half goes into the coefficient
-    const real hwdg = real(0.5) * wdg;
+    // exactly (a power-of-two scale), so the pair's mean normal is left unhalved, as are the
+    // means inside volume_flux, and the quarter goes into the coefficient
+    const real qwdg = real(0.25) * wdg;
 
     // flux differencing: every symmetric pair once (split form, zero diagonal)
 #pragma unroll
@@ -772,7 +786,7 @@ rhs_kernel(const DgArgs a, const KConst kc) {
         volume_flux<real, DIM, NSP>(vf, q[ni], vi, q[(1 + DIM) * NP + ni], q[(2 + DIM) * NP + ni], ui,
                                     q[nl], vl, q[(1 + DIM) * NP + nl], q[(2 + DIM) * NP + nl], ul,
                                     nrm, kc.inv_gm1, kc.pref, F);
-        const real cil = hwdg * B.D2[i * N1 + l], cli = hwdg * B.D2[l * N1 + i];
+        const real cil = qwdg * B.D2[i * N1 + l], cli = qwdg * B.D2[l * N1 + i];
         axpy<NV>(acc[i], cil, F);
         axpy<NV>(acc[l], cli, F);
       }
@@ -811,8 +825,10 @@ rhs_kernel(const DgArgs a, const KConst kc) {
         Lq.p = Lq.pp + kc.pref;
         Rq.p = Rq.pp + kc.pref;
         if (NSP == 1) {
-          Lq.c = RealOps<real>::sqrt_(kc.gamma * Lq.p * RealOps<real>::rcp(Lq.rho));
-          Rq.c = RealOps<real>::sqrt_(kc.gamma * Rq.p * RealOps<real>::rcp(Rq.rho));
+          Lq.cc = kc.gamma * Lq.p * RealOps<real>::rcp(Lq.rho);
+          Lq.c = RealOps<real>::sqrt_(Lq.cc);
+          Rq.cc = kc.gamma * Rq.p * RealOps<real>::rcp(Rq.rho);
+          Rq.c = RealOps<real>::sqrt_(Rq.cc);
         } else {
           Lq.c = spc[e * L::SPC + NP + nl];
           Rq.c = spc[e * L::SPC + NP + nr];
@@ -1434,7 +1450,8 @@ gradient_kernel(const DgArgs a, const KConst kc) {
       // boundary faces get their lifting from boundary_lift_kernel: here a valid address
       // (the own element) and a zero weight, without a branch
       const real* un = gu + (int64_t)(nb >= 0 ? nb : eg) * NV * NP + nnode;
-      const real keep = nb >= 0 ? real(1) : real(0);
+      // the lifted jump W* - W is half of the jump to the neighbour
+      const real lift = nb >= 0 ? (side ? real(0.5) * B.iw[N] : real(-0.5) * B.iw[0]) : real(0);
       real rn = 0;
 #pragma unroll
       for (int k = 0; k < NSP; ++k) rn += un[k * NP];
@@ -1447,9 +1464,8 @@ gradient_kernel(const DgArgs a, const KConst kc) {
       Wn[DIM] = kc.gm1 * (un[(NSP + DIM) * NP] - real(0.5) * ke) * irn;
 #pragma unroll
       for (int c = 0; c < NW; ++c) {
-        real ws = real(0.5) * (Wl[i][c] + Wn[c]);
-        if (side) G[N][c] += keep * B.iw[N] * (ws - Wl[N][c]);
-        else G[0][c] -= keep * B.iw[0] * (ws - Wl[0][c]);
+        if (side) G[N][c] += lift * (Wn[c] - Wl[N][c]);
+        else G[0][c] += lift * (Wn[c] - Wl[0][c]);
       }
     }
     real* g = sg + e * L::SG + d * NW * NP;
@@ -1460,7 +1476,7 @@ gradient_kernel(const DgArgs a, const KConst kc) {
   }
   __syncthreads();
   trigger();
-  // physical gradients G_x = (1/J) sum_d Ja^d_x Q_d; written as they are (grad_mode 1) or
+  // physical gradients G_x = (1/J) sum_d Ja^d_x Q_d (G without the 1/J); written as they are (grad_mode 1) or
   // turned into the contravariant viscous fluxes sum_x Ja^d_x f^v_x(G; v, mu(T)) that the
   // right-hand-side kernel consumes (grad_mode 0)
   real* out = (real*)a.gradW;
@@ -1476,20 +1492,20 @@ gradient_kernel(const DgArgs a, const KConst kc) {
         real acc = 0;
 #pragma unroll
         for (int d = 0; d < DIM; ++d) acc += jn[(d * DIM + x) * NP] * sg[e * L::SG + (d * NW + c) * NP + pn];
-        G[x][c] = acc * ij;
+        G[x][c] = acc;
       }
     real* o = out + (e0 + e) * DIM * NW * NP + node;
     if (a.grad_mode) {
 #pragma unroll
       for (int x = 0; x < DIM; ++x)
 #pragma unroll
-        for (int c = 0; c < NW; ++c) o[(x * NW + c) * NP] = G[x][c];
+        for (int c = 0; c < NW; ++c) o[(x * NW + c) * NP] = G[x][c] * ij;
       continue;
     }
     real vv[DIM];
 #pragma unroll
     for (int c = 0; c < DIM; ++c) vv[c] = sw[e * L::SW + c * NP + pn];
-    real mu_n = kc.mu, kap_n = kc.kap;
+    real mu_n = kc.mu * ij, kap_n = kc.kap * ij;  // the flux is linear in the gradient: 1/J goes here
     if (kc.suth_s > real(0)) {
       const real r = sutherland_ratio(sw[e * L::SW + DIM * NP + pn], kc.suth_s, kc.suth_c1, kc.suth_irt);
       mu_n *= r;
