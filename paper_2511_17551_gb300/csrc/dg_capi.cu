@@ -11,6 +11,7 @@
 #include <utility>
 
 #include "../../include/dg.h"
+#include "dg_cvt.cuh"
 #include "dg_internal.h"
 #include "dg_thermo.h"
 
@@ -180,16 +181,13 @@ __global__ void cvt_back_kernel(const T* a, double* b, int64_t n) {
 // compensated FP32 state of the mixed form: u = hi + lo, hi = fl32(u), lo = fl32(u - hi)
 __global__ void split_kernel(const double* a, float* hi, float* lo, int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const float h = (float)a[i];
-    hi[i] = h;
-    lo[i] = (float)(a[i] - (double)h);
-  }
+       i += (int64_t)gridDim.x * blockDim.x)
+    split_f64(a[i], hi[i], lo[i]);
 }
 __global__ void merge_kernel(const float* hi, const float* lo, double* b, int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
-    b[i] = (double)hi[i] + (double)lo[i];
+    b[i] = merge_f64(hi[i], lo[i]);
 }
 // The same two conversions for 16-byte aligned buffers, built for the host link (a
 // page-locked host buffer read or written in place): pairs of values as 16-byte accesses,
@@ -205,16 +203,20 @@ __global__ void split_kernel_x4(const double2* a, float2* hi, float2* lo, int64_
     for (int j = 0; j < 4; ++j) v[j] = a[i + j * st];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const float hx = (float)v[j].x, hy = (float)v[j].y;
-      hi[i + j * st] = make_float2(hx, hy);
-      lo[i + j * st] = make_float2((float)(v[j].x - (double)hx), (float)(v[j].y - (double)hy));
+      float2 h, l;
+      split_f64(v[j].x, h.x, l.x);
+      split_f64(v[j].y, h.y, l.y);
+      hi[i + j * st] = h;
+      lo[i + j * st] = l;
     }
   }
   for (; i < n2; i += st) {
     const double2 v = a[i];
-    const float hx = (float)v.x, hy = (float)v.y;
-    hi[i] = make_float2(hx, hy);
-    lo[i] = make_float2((float)(v.x - (double)hx), (float)(v.y - (double)hy));
+    float2 h, l;
+    split_f64(v.x, h.x, l.x);
+    split_f64(v.y, h.y, l.y);
+    hi[i] = h;
+    lo[i] = l;
   }
 }
 __global__ void merge_kernel_x4(const float2* hi, const float2* lo, double2* b, int64_t n2) {
@@ -229,11 +231,11 @@ __global__ void merge_kernel_x4(const float2* hi, const float2* lo, double2* b, 
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      b[i + j * st] = make_double2((double)h[j].x + (double)l[j].x, (double)h[j].y + (double)l[j].y);
+      b[i + j * st] = make_double2(merge_f64(h[j].x, l[j].x), merge_f64(h[j].y, l[j].y));
   }
   for (; i < n2; i += st) {
     const float2 hh = hi[i], ll = lo[i];
-    b[i] = make_double2((double)hh.x + (double)ll.x, (double)hh.y + (double)ll.y);
+    b[i] = make_double2(merge_f64(hh.x, ll.x), merge_f64(hh.y, ll.y));
   }
 }
 // split / merge of n values: the 16-byte kernels where every pointer allows, the odd last
@@ -264,15 +266,15 @@ void launch_merge(const float* hi, const float* lo, double* dst, int64_t n, cuda
 }
 
 // one-gas primitive (rho, v, p) -> conserved, written in the form precision (lo: the FP32 form's
-// compensation part, or null).  Bound by memory: (dim + 2) doubles in, as many bytes out.  The values
-// stay in registers (compile-time dim; with a run-time one they went through local memory), and
-// the 64-bit division that splits the node index is one per CTA and pass: 32^3 elements, N = 3,
-// a call 162 -> 147 us (the conversions of the hi / lo split on the FP64 pipe are what is left).
+// compensation part, or null).  (dim + 2) doubles in, as many bytes out; bound by the FP64 pipe, about
+// three operations a value.  The values stay in registers (compile-time dim; with a run-time one they
+// went through local memory), the 64-bit division that splits the node index is one per CTA and
+// pass, and 1 / (gamma - 1) comes from the host: 32^3 elements, N = 3, a call 157 -> 111 -> 71 us, the
+// second step by the conversions of the split in integer work.
 template <typename T, int DIM>
 __global__ void __launch_bounds__(256) prim2cons_kernel(const double* w, T* u, float* lo, int64_t K, int np,
-                                                        double gamma) {
+                                                        double igm1) {
   constexpr int NV = DIM + 2;
-  const double igm1 = 1.0 / (gamma - 1.0);
   for (int64_t base = blockIdx.x * (int64_t)256; base < K * np; base += gridDim.x * (int64_t)256) {
     const int64_t k0 = base / np;
     const unsigned off = (unsigned)(base - k0 * np) + threadIdx.x, dk = off / (unsigned)np;
@@ -290,17 +292,20 @@ __global__ void __launch_bounds__(256) prim2cons_kernel(const double* w, T* u, f
     c[1 + DIM] = c[1 + DIM] * igm1 + 0.5 * c[0] * ke;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      const T h = (T)c[v];
-      u[at + v * np] = h;
-      if (lo) lo[at + v * np] = (float)(c[v] - (double)h);
+      if constexpr (sizeof(T) == 4) {
+        if (lo) split_f64(c[v], u[at + v * np], lo[at + v * np]);
+        else u[at + v * np] = f64_to_f32(c[v]);
+      } else {
+        u[at + v * np] = c[v];
+      }
     }
   }
 }
 template <typename T>
 void launch_prim2cons(const double* w, T* u, float* lo, int64_t K, int dim, int np, double gamma, unsigned grid,
                       cudaStream_t st) {
-  if (dim == 3) prim2cons_kernel<T, 3><<<grid, 256, 0, st>>>(w, u, lo, K, np, gamma);
-  else prim2cons_kernel<T, 2><<<grid, 256, 0, st>>>(w, u, lo, K, np, gamma);
+  if (dim == 3) prim2cons_kernel<T, 3><<<grid, 256, 0, st>>>(w, u, lo, K, np, 1.0 / (gamma - 1.0));
+  else prim2cons_kernel<T, 2><<<grid, 256, 0, st>>>(w, u, lo, K, np, 1.0 / (gamma - 1.0));
 }
 
 // FP64 domain integrals, per block partial sums (deterministic: the grid depends on K alone, fixed

@@ -20,6 +20,7 @@
 #include <string.h>
 
 #include "dg_dd.cuh"
+#include "dg_cvt.cuh"
 #include "dg_internal.h"
 #include "dg_launch.cuh"
 #include "dg_thermo.h"
@@ -224,7 +225,7 @@ __global__ void __launch_bounds__(256, 3) thermo_mixed_kernel(const float* u, in
 // (rho_s, v, T) -> conserved; seeds the temperature cache Tc, or (boundary states) gives (p, c).  The
 // energy is summed over the species as rho e = sum_k T^k sum_s rho_s c_sk: 46 FP64 operations a node
 // (the pipe bounds the kernel) instead of about 150 with mass fractions and (p, c), which the
-// temperature solve of every later evaluation forms anew: 1.73 M nodes 462 -> 209 us a call.
+// temperature solve of every later evaluation forms anew: 1.73 M nodes 457 -> 189 us a call.
 template <typename T>
 __global__ void __launch_bounds__(256) thermo_prim2cons_kernel(const double* w, T* u, int64_t K, int np, int dim,
                                                                const double* cf, double* Tc, T* pc) {
@@ -244,17 +245,17 @@ __global__ void __launch_bounds__(256) thermo_prim2cons_kernel(const double* w, 
     for (int s = 0; s < NSPEC; ++s) {
       r[s] = ww[s * np];
       rho += r[s];
-      uu[s * np] = (T)r[s];
+      uu[s * np] = narrow<T>(r[s]);
     }
     double ke = 0.0;
     for (int d = 0; d < dim; ++d) {
       const double v = ww[(NSPEC + d) * np];
-      uu[(NSPEC + d) * np] = (T)(rho * v);
+      uu[(NSPEC + d) * np] = narrow<T>(rho * v);
       ke += v * v;
     }
     const double Tk = ww[(NSPEC + dim) * np];
     build_poly<double>(cf, r, P);
-    uu[(NSPEC + dim) * np] = (T)(P.e(Tk) + 0.5 * rho * ke);
+    uu[(NSPEC + dim) * np] = narrow<T>(P.e(Tk) + 0.5 * rho * ke);
     if (Tc) Tc[k * np + node] = Tk;
     if (pc) {
       const double p = P.Rmix * Tk, cv = P.cv(Tk);
