@@ -234,8 +234,10 @@ static_assert(sizeof(ChemTab32) < 16 * 1024, "a kernel argument");
 // difference comes from delta itself.  Measured against FP64 on states with rates from cold to 9000 K
 // and after 50 steps: the same relative L2 to three digits (2.5e-8, the rounding of the result).
 // What bounds it: about 200 FP64 operations and 8,000 others per node, on two pipes; 1,063 FP64
-// operations before.  4.6 M nodes: 10.17 -> 2.28 ms.  All of it in pairs, logarithms, g and delta too,
-// ran in 1.20 ms but missed the FP64 source by a tenfold larger maximum near equilibrium.
+// operations before.  4.6 M nodes: 10.17 -> 2.28 ms, and 1.74 ms since the conversions to and from
+// pairs are integer work (as instructions they took a quarter of the FP64 pipe's time).  All of it in
+// pairs, logarithms, g and delta too, missed the FP64 source by a tenfold larger maximum near
+// equilibrium.
 // Returns false where the pairs do not hold (a concentration that is not between 1e-24 and
 // 1e6 mol/cm^3, zero and negative ones among them, or a result that is not finite); the caller
 // then evaluates the node in FP64.
@@ -511,10 +513,15 @@ chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, co
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const int nv = NSPEC + dim + 1;
   const int64_t total = K * np;
-  if (cmode != 2 && blockIdx.x == 0 && threadIdx.x == 0) stats[2] = 0;  // chem_fallback_kernel's tile counter
+  // behind the wait for the preceding kernel; tables and weights, which no kernel writes, come before it
+  auto enter = [&]() {
+    pdl_wait();
+    if (cmode != 2 && blockIdx.x == 0 && threadIdx.x == 0) stats[2] = 0;  // chem_fallback_kernel's tile counter
+  };
   if ((int)blockIdx.x < checks) {
     typename Form::Tab& tb = *reinterpret_cast<typename Form::Tab*>(smem_raw);
     Form::stage(tb, exp2);
+    enter();
     const int64_t t = blockIdx.x * (int64_t)dgtc5::THREADS + threadIdx.x;
     if (t * 32 >= total || (cmode == 1 && !trust[t])) return;
     typename ChemForm<T>::step dt;
@@ -538,6 +545,7 @@ chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, co
   if (sizeof(T) == 4)
     for (int j = threadIdx.x; j < dgdd::EXP_TAB; j += dgtc5::THREADS) e2[j] = exp2[j];
   dgtc5::load_weights<10, CHEM_NR>(s, mlp->w);
+  enter();
   __syncthreads();
   const float dt = dtp ? (float)*dtp : 0.f;
   auto prod = [&](int64_t i, float* x, int) {
@@ -644,6 +652,7 @@ chem_fallback_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, c
   typedef typename ChemForm<T>::type Form;
   __shared__ typename Form::Tab tb;
   Form::stage(tb, exp2);
+  pdl_wait();
   const int nv = NSPEC + dim + 1;
   const int lane = threadIdx.x & 31;
   const int64_t total = K * np, ntiles = (total + 31) / 32;
@@ -774,6 +783,7 @@ chem_refresh_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, co
   typedef typename ChemForm<T>::type Form;
   __shared__ typename Form::Tab tb;
   Form::stage(tb, exp2);
+  pdl_wait();
   const int nv = NSPEC + dim + 1;
   const int64_t total = K * np;
   typename ChemForm<T>::step dt;
@@ -946,30 +956,28 @@ static cudaError_t chem_learned(DgThermo* th, const T* u, const double* dt_dev, 
   const unsigned g1 = (unsigned)(tiles < 152 * 5 ? tiles : 152 * 5);
   if (refresh) {
     if (!th->chem_corr || !th->chem_trust) return cudaErrorInvalidValue;
-    k1<<<g1, dgtc5::THREADS, smem, s>>>(u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr, tab, e2, m,
-                                        dt_dev, (T*)th->src, th->chem_flags, th->chem_corr, th->chem_trust, 2, 0,
-                                        NULL, 0, NULL);
-    chem_refresh_kernel<T><<<grid_of(ntiles * 32), 128, 0, s>>>(u, th->T, th->K, th->np, th->dim,
-                                                                th->species_raw, th->reac, th->nr, tab, e2, m, dt_dev,
-                                                                (T*)th->src, th->chem_corr, th->chem_flags,
-                                                                th->chem_trust);
-    e = cudaGetLastError();
+    e = launch_pdl(k1, g1, dgtc5::THREADS, smem, s, u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr,
+                   tab, e2, m, dt_dev, (T*)th->src, th->chem_flags, th->chem_corr, th->chem_trust, 2, 0, (T*)NULL, 0,
+                   (unsigned long long*)NULL);
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(chem_refresh_kernel<T>, grid_of(ntiles * 32), 128, 0, s, u, th->T, th->K, th->np, th->dim,
+                   th->species_raw, th->reac, th->nr, tab, e2, m, dt_dev, (T*)th->src, th->chem_corr, th->chem_flags,
+                   th->chem_trust);
     if (e == cudaSuccess) th->corr_valid = 1;
     return e;
   }
   const int cmode = th->chem_corr && th->chem_trust && th->corr_valid ? 1 : 0;
   const unsigned checks = (unsigned)((ntiles + dgtc5::THREADS - 1) / dgtc5::THREADS);
   const uint64_t call = th->chem_calls++;
-  k1<<<checks + g1, dgtc5::THREADS, smem, s>>>(u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr,
-                                               tab, e2, m, dt_dev, (T*)th->src, th->chem_flags, th->chem_corr,
-                                               th->chem_trust, cmode, (int)checks, (T*)th->chem_sampled, call,
-                                               th->chem_stats);
+  e = launch_pdl(k1, checks + g1, dgtc5::THREADS, smem, s, u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac,
+                 th->nr, tab, e2, m, dt_dev, (T*)th->src, th->chem_flags, th->chem_corr, th->chem_trust, cmode,
+                 (int)checks, (T*)th->chem_sampled, call, th->chem_stats);
+  if (e != cudaSuccess) return e;
   int64_t g3 = (ntiles + 3) / 4;
   if (g3 > 152 * 5) g3 = 152 * 5;
-  chem_fallback_kernel<T><<<(unsigned)g3, 128, 0, s>>>(u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac,
-                                                       th->nr, tab, e2, m, dt_dev, (T*)th->src, th->chem_flags,
-                                                       (const T*)th->chem_sampled, call, th->chem_stats);
-  return cudaGetLastError();
+  return launch_pdl(chem_fallback_kernel<T>, (unsigned)g3, 128, 0, s, u, th->T, th->K, th->np, th->dim, th->species_raw,
+                    th->reac, th->nr, tab, e2, m, dt_dev, (T*)th->src, th->chem_flags, (const T*)th->chem_sampled, call,
+                    th->chem_stats);
 }
 
 cudaError_t dg_chem_source(DgThermo* th, const void* u, int f32, const double* dt_dev, int refresh,

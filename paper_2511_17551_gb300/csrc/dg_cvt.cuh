@@ -33,3 +33,21 @@ __device__ __forceinline__ void split_f64(double x, float& hi, float& lo) {
   lo = f64_to_f32(x - f32_to_f64(hi));
 }
 __device__ __forceinline__ double merge_f64(float hi, float lo) { return f32_to_f64(hi) + f32_to_f64(lo); }
+
+// Without a slow path, for the middle of heavier kernels (the call would cost them registers):
+// magnitudes below 2^-126 become zeros, and a double of 2^128 and more becomes NaN.
+__device__ __forceinline__ float f64_to_f32_mid(double x) {
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x), a = h & 0x7fffffffu;
+  unsigned m = __funnelshift_l(l, a - 0x38000000u, 3);
+  m += ((l << 3) + (m & 1u)) > 0x80000000u;
+  m = a < 0x38100000u ? 0u : m;
+  m = a >= 0x47f00000u ? 0x7fffffffu : m;
+  return __uint_as_float(m | (h & 0x80000000u));
+}
+__device__ __forceinline__ double f32_to_f64_mid(float x) {
+  const unsigned b = __float_as_uint(x), a = b & 0x7fffffffu;
+  const bool tiny = a < 0x00800000u;
+  unsigned h = tiny ? 0u : (a >> 3) + 0x38000000u;
+  h = a >= 0x7f800000u ? h | 0x7ff00000u : h;  // infinite, NaN
+  return __hiloint2double((int)(h | (b & 0x80000000u)), tiny ? 0 : (int)(a << 29));
+}

@@ -12,6 +12,7 @@
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
+#include "dg_cvt.cuh"
 
 namespace dgdd {
 
@@ -62,12 +63,27 @@ DG_HD dd make(float h, float l) {
   r.l = l;
   return r;
 }
+// conversions between the two (dg_cvt.cuh: integer work on the device)
+DG_HD float narrow(double x) {
+#ifdef __CUDA_ARCH__
+  return f64_to_f32_mid(x);
+#else
+  return (float)x;
+#endif
+}
+DG_HD double widen(float x) {
+#ifdef __CUDA_ARCH__
+  return f32_to_f64_mid(x);
+#else
+  return (double)x;
+#endif
+}
 // the FP64 number as a pair
 DG_HD dd from_double(double x) {
-  const float h = (float)x;
-  return make(h, (float)(x - (double)h));
+  const float h = narrow(x);
+  return make(h, narrow(x - widen(h)));
 }
-DG_HD double to_double(dd a) { return (double)a.h + (double)a.l; }
+DG_HD double to_double(dd a) { return widen(a.h) + widen(a.l); }
 DG_HD dd neg(dd a) { return make(-a.h, -a.l); }
 
 DG_HD dd two_sum(float a, float b) {
@@ -193,7 +209,7 @@ DG_HD dd log_(dd x, const dd* tab, double* sum64 = nullptr) {
   const float p = fmul(x.h, E.h);
   const float pe = ffma(x.l, E.h, ffma(x.h, E.l, ffma(x.h, E.h, -p)));
   const float z = fsub(p, 1.0f), t = ffma(fmul(-0.5f, z), z, pe);
-  if (sum64) *sum64 = (double)y0 + ((double)z + (double)t);
+  if (sum64) *sum64 = widen(y0) + (widen(z) + widen(t));
   const dd s = two_sum(y0, z);
   return quick_two_sum(s.h, fadd(s.l, t));
 }

@@ -63,6 +63,12 @@ __device__ __forceinline__ void build_poly(const R* cf, const R* Y, Poly<R>& P) 
 }
 
 __device__ __forceinline__ double clampT(double T) { return T < 200.0 ? 200.0 : (T > 1e4 ? 1e4 : T); }
+// 200 <= T <= 1e4, false for NaN: positive doubles order as their bits do (200.0 is 0x40690000 00000000,
+// 1e4 0x40c38800 00000000)
+__device__ __forceinline__ bool in_fit_range(double T) {
+  const unsigned h = (unsigned)__double2hiint(T);
+  return h >= 0x40690000u && (h < 0x40c38800u || (h == 0x40c38800u && __double2loint(T) == 0));
+}
 __device__ __forceinline__ float clampTf(float T) { return T < 200.f ? 200.f : (T > 1e4f ? 1e4f : T); }
 
 // FP64 Newton from T; returns true on convergence
@@ -136,10 +142,10 @@ __device__ __noinline__ bool newton64_node(const float* uu, int np, int dim, con
 // double-FP32 pairs (dg_dd.cuh): the FP32 state is exact in them, e - b0 keeps 46 bits through
 // the cancellation of the formation energies, and the polynomial takes the FP32-rounded
 // temperature coefficients (their rounding moves e by ~1e-7 relative, i.e. T by ~1e-4 K, as it
-// did with the residual in FP64).  Nothing in the common path touches the FP64 pipe but the
-// conversions of the cached temperature; 68 FP64 instructions a node bound the kernel before.
-// Bytes per node: 36 of state, 16 of T, 8 of (p, c).  1.73 M nodes: 193 -> 55 us (1.9 TB/s), 4.6 M:
-// 500 -> 113 us (2.4 TB/s); the same distance to the FP64 solution (1.6e-7, the coefficients').
+// did with the residual in FP64).  Nothing in the common path touches the FP64 pipe but one
+// addition; 68 FP64 instructions a node bound the kernel before.
+// Bytes per node: 36 of state, 16 of T, 8 of (p, c).  1.73 M nodes: 193 -> 45 us (2.3 TB/s), 4.6 M:
+// 500 -> 101 us (2.7 TB/s); the same distance to the FP64 solution (1.6e-7, the coefficients').
 template <int NP, int DIM>
 __global__ void __launch_bounds__(256, 3) thermo_mixed_kernel(const float* u, int64_t K, const double* cf,
                                                            const float* cf32, double* Tc, float* pc,
@@ -188,8 +194,8 @@ __global__ void __launch_bounds__(256, 3) thermo_mixed_kernel(const float* u, in
 #pragma unroll
     for (int s = 0; s < NSPEC; ++s) Y[s] = r[s] * ir.h;
     build_poly<float>(c32, Y, P);
-    if (!(Tk >= 200.0 && Tk <= 1e4)) Tk = 1000.0;
-    float Tf = (float)Tk;
+    if (!in_fit_range(Tk)) Tk = 1000.0;
+    float Tf = dgdd::narrow(Tk);
     bool conv = false;
     // (below 1e-12 kg/m^3 the products' low parts leave FP32's range: FP64)
     for (int it = 0; it < 12 && rho.h > 1e-12f; ++it) {
@@ -215,7 +221,7 @@ __global__ void __launch_bounds__(256, 3) thermo_mixed_kernel(const float* u, in
     if (ok && !conv) ok = newton64_node(uu, NP, DIM, cf, T64);
     if (!ok) latch(status, DG_ST_NEWTON, k);
     Tc[k * NP + node] = T64;
-    const float Tq = (ok && !conv) ? (float)T64 : T.h;
+    const float Tq = (ok && !conv) ? dgdd::narrow(T64) : T.h;
     const float pf = rho.h * P.Rmix * Tq, cvf = P.cv(Tq);
     pc[(k * 2 + 0) * NP + node] = pf;
     pc[(k * 2 + 1) * NP + node] = sqrtf((cvf + P.Rmix) / cvf * pf / rho.h);
