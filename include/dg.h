@@ -197,7 +197,8 @@ dg_status dg_get_temperature(dg_ctx* ctx, double* T);
 /* ---- learned surrogates (no counterpart in the paper).  Both are a perceptron
  * 7 -> 64 -> 64 -> n_out with the tanh form of GELU after the hidden layers, evaluated
  * with BF16 tensor-core MMAs (FP32 accumulation) and always checked against the plain
- * FP64 computation they replace, which remains the fallback.  Parameter vector (FP32,
+ * computation they replace, which remains the fallback (the source: FP64 in the FP64 form;
+ * in the mixed form FP64 thermodynamics and kinetics in pairs of FP32 values, 48 bits).  Parameter vector (FP32,
  * P = dg_mlp_nparams(n_out)): W1[64][7], b1[64], W2[64][64], b2[64], W3[n_out][64],
  * b3[n_out].
  *
@@ -216,7 +217,7 @@ dg_status dg_get_temperature(dg_ctx* ctx, double* T);
  *   mass-balanced (|sum omega| <= tol_mass sum |omega| + floor), every node's learned
  *   update positive (rho_s + dt S_s >= 0, dt the running step), and, at one node per tile drawn
  *   anew each evaluation, |S_learned - S_plain| <= tol_check sum_s |S_plain| + floor for
- *   every species; rejected tiles are recomputed with the plain FP64 source.  Accepted
+ *   every species; rejected tiles are recomputed with the plain source.  Accepted
  *   rates are projected onto exact mass balance, omega_s -= |omega_s| sum omega / sum|omega|. */
 enum { DG_SURROGATE_TEMPERATURE = 0, DG_SURROGATE_SOURCE = 1 };
 enum {
@@ -242,7 +243,7 @@ enum {
 dg_status dg_set_surrogate(dg_ctx* ctx, int which, const float* params, const double* stats);
 
 /* Plain correction of the learned source (reacting contexts).  period 0 (the default)
- * switches it off.  period k >= 1: a refresh evaluation takes the plain FP64 source at
+ * switches it off.  period k >= 1: a refresh evaluation takes the plain source at
  * every node and stores per node the plain rates minus the network's decoded rates
  * (omega_s - omega^_s and jpi_s - jpi'_s, jpi' the decoded jpi before its clamp at 0;
  * FP32, 40 bytes per node, allocated here); the learned evaluations that follow add these

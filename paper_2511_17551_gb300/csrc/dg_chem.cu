@@ -1,7 +1,7 @@
 // Finite-rate chemistry source on the device (appendix, Chemical Kinetics: Eqs. nrp,
 // forward_rate, backward, kedef, calc_prod), one thread per node: in FP64 in the FP64 form
-// (chem_node), in double-FP32 arithmetic in the mixed form (chem_node_dd), whose source is
-// rounded to FP32 in either case.
+// (chem_node); in the mixed form (chem_node_dd) the thermodynamics in FP64 and the kinetics in
+// double-FP32 pairs, the source rounded to FP32.
 //
 // Concentrations c_s = 1e-6 rho_s / W_s (mol/cm^3, the units of Park-type constants);
 // k_f = exp(ln A + beta ln T - theta/T); k_b = k_f / K_c with
@@ -409,7 +409,7 @@ chem_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, const doub
 // Acceptance, per tile of 32 nodes (one warp): every node inside the training box, every
 // node's raw rates mass-balanced (|sum omega| <= tol_mass sum|omega| + floor), every
 // node's learned update positive (rho_s + dt S_s >= 0), and one sampled node per tile
-// (moved each call) within tol_check of the plain FP64 source; otherwise the tile's source
+// (moved each call) within tol_check of the plain source; otherwise the tile's source
 // is recomputed plainly.  Accepted rates are projected onto exact mass balance:
 // omega_s -= |omega_s| sum(omega) / sum|omega|.
 // With a refresh period (plain correction): a refresh evaluation takes the plain source at

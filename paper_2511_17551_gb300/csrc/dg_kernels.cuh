@@ -6,16 +6,16 @@
 //   phase A  coalesced (16-byte) copy of the elements' conserved state, metric
 //            terms and 1/J into shared memory; per-node primitives (rho, v, p,
 //            rho/p) computed once; for Navier-Stokes, the viscous fluxes f^v_x.
-//   phase B1 one thread per grid line (direction d, line m): every symmetric pair
+//   phase B  one thread per grid line (direction d, line m): every symmetric pair
 //            (i < l) of the line is evaluated ONCE with the two-point flux and
 //            added to both end points with 2 D_il and 2 D_li in registers (split
 //            form with zero diagonal, Eqs. fluxdiff / fluxdiffcons, so no self-flux
 //            is ever formed), plus the subcell FV fluxes of blended elements
 //            (Eq. fluxes_discrete_with_fv) and the BR1 viscous volume term (Eq.
 //            auxstrongf); each line stores its N+1 node sums once.
-//   phase B2 one thread per face node: interface flux from the neighbour's trace
-//            (Eqs. riemann_problem1-3) or the boundary state, lifted onto the face
-//            node, plus the averaged viscous interface flux.
+//            Before its pairs each line takes the interface fluxes at its two end
+//            nodes, from the neighbour's trace (Eqs. riemann_problem1-3) or the boundary
+//            state, lifted onto those nodes, plus the averaged viscous interface flux.
 //   phase C  one thread per node: sum the DIM line contributions in a fixed
 //            order, scale by -1/J, and either store du/dt or apply the
 //            2N-storage Runge-Kutta update (and the wave-speed maximum of the
