@@ -9,6 +9,7 @@
 #include <string.h>
 
 #include "../../include/dg.h"
+#include "dg_launch.cuh"
 #include "dg_mlp.cuh"
 
 namespace {
@@ -120,6 +121,7 @@ __global__ void count_le_kernel(const double* Y, int64_t n, int d, int c0, int n
 }
 
 __global__ void gather_rows_kernel(const float* X, int d, const int64_t* idx, int64_t m, float* out) {
+  pdl_wait();
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < m * d; q += (int64_t)gridDim.x * blockDim.x)
     out[q] = X[idx[q / d] * d + q % d];
 }
@@ -295,8 +297,9 @@ dg_status dg_gather_rows(const float* X, int d, const int64_t* idx, int64_t m, f
   if (!X || !idx || !out || d < 1 || m < 1) return DG_EINVAL;
   int64_t g = (m * d + 255) / 256;
   if (g > 152 * 32) g = 152 * 32;
-  gather_rows_kernel<<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(X, d, idx, m, out);
-  return cudaGetLastError() == cudaSuccess ? DG_OK : DG_ECUDA;
+  return launch_pdl(gather_rows_kernel, (unsigned)g, 256, 0, (cudaStream_t)stream, X, d, idx, m, out) == cudaSuccess
+             ? DG_OK
+             : DG_ECUDA;
 }
 
 dg_status dg_mlp_loss(const float* params, int n_out, const float* X, const float* t, int64_t n, double* loss,

@@ -14,7 +14,8 @@
 // 14 % against there, since the next kernel's CTAs then take the places that their own CTAs leave
 // and lie unevenly on the SMs.  In FP64, where the FP64 pipe of an SM bounds its CTAs, that weighs
 // more than the overlap (8^3: 2.61 -> 3.13 ms), so FP64 kernels do not trigger at all: only
-// the launch itself is hidden (2.61 -> 2.49 ms).
+// the launch itself is hidden (2.61 -> 2.49 ms).  Nor do the training kernels, one wave of CTAs each: an
+// iteration of gathers, gradient and Adam 36 -> 25 us.
 #pragma once
 #include <cuda_runtime.h>
 

@@ -16,6 +16,7 @@
 
 #include "../../include/dg.h"
 #include "dg_internal.h"
+#include "dg_launch.cuh"
 #include "dg_mlp.cuh"
 #include "dg_mlp_tc5.cuh"
 #include "dg_thermo.h"
@@ -310,7 +311,7 @@ __device__ __forceinline__ void tile_2x4(const float* a0, const float* a1, const
 // its transpose, its gradient) are 2 x 4 and 4 x 4 register tiles over 256 threads with 16-byte
 // shared-memory reads; the gradient sums stay in registers over the tiles.  With 64 threads, one
 // per unit, and every operand read 4 bytes at a time, a fitting iteration (two
-// gathers, this, Adam) with a batch of 4,096 and ten outputs took 88 us, now 36; what is left is the
+// gathers, this, Adam) with a batch of 4,096 and ten outputs took 88 us, then 36, and 25 since the launches overlap (dg_launch.cuh); what is left is the
 // chain of eight barriers of one tile per CTA (128 CTAs) and the launches.
 __global__ void __launch_bounds__(TT) mlp_grad_kernel(const float* P, int no, const float* X, const float* t, int B,
                                                       float* partial) {
@@ -318,6 +319,7 @@ __global__ void __launch_bounds__(TT) mlp_grad_kernel(const float* P, int no, co
   TrainSmem& S = *reinterpret_cast<TrainSmem*>(raw);
   const int tid = threadIdx.x;
   const int OW3 = dg_mlp_off_w3(), OB3 = dg_mlp_off_b3(no), NPAR = dg_mlp_np(no);
+  pdl_wait();
 #pragma unroll 4
   for (int q = tid; q < NH * NH; q += TT) {
     const float w = P[OFF_W2 + q];
@@ -492,6 +494,7 @@ __global__ void __launch_bounds__(256) mlp_reduce_adam_kernel(const float* parti
   __shared__ float part[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = blockIdx.x * 32 + lane;
   float s = 0.f;
+  pdl_wait();
   if (q <= npar) {
 #pragma unroll 8
     for (int b = w; b < nb; b += 8) s += partial[(int64_t)b * (npar + 1) + q];
@@ -687,8 +690,7 @@ static dg_status grad_common(const float* P, int no, const float* X, const float
   if (cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return DG_ECUDA;
-  mlp_grad_kernel<<<nb, TT, smem, st>>>(P, no, X, t, B, ws);
-  if (cudaGetLastError() != cudaSuccess) return DG_ECUDA;
+  if (launch_pdl(mlp_grad_kernel, nb, TT, smem, st, P, no, X, t, B, ws) != cudaSuccess) return DG_ECUDA;
   *nb_out = nb;
   return DG_OK;
 }
@@ -701,9 +703,10 @@ dg_status dg_mlp_grad(const float* params, int n_out, const float* X, const floa
   if (r != DG_OK) return r;
   if (!grad) return DG_EINVAL;
   const int npar = dg_mlp_np(n_out);
-  mlp_reduce_adam_kernel<<<(npar + 1 + 31) / 32, 256, 0, st>>>(workspace, nb, npar, grad, NULL, NULL, NULL, 0,
-                                                                 0.f, 0.f, 0.f, 0.f, loss);
-  return cudaGetLastError() == cudaSuccess ? DG_OK : DG_ECUDA;
+  return launch_pdl(mlp_reduce_adam_kernel, (npar + 1 + 31) / 32, 256, 0, st, workspace, nb, npar, grad, (float*)NULL,
+                    (float*)NULL, (float*)NULL, 0, 0.f, 0.f, 0.f, 0.f, loss) == cudaSuccess
+             ? DG_OK
+             : DG_ECUDA;
 }
 
 dg_status dg_mlp_train_step(float* params, int n_out, float* m, float* v, const float* X, const float* t,
@@ -715,9 +718,10 @@ dg_status dg_mlp_train_step(float* params, int n_out, float* m, float* v, const 
   dg_status r = grad_common(params, n_out, X, t, batch, workspace, ws_bytes, st, &nb);
   if (r != DG_OK) return r;
   const int npar = dg_mlp_np(n_out);
-  mlp_reduce_adam_kernel<<<(npar + 1 + 31) / 32, 256, 0, st>>>(workspace, nb, npar, NULL, params, m, v, step,
-                                                                 lr, 0.9f, 0.999f, 1e-8f, loss);
-  return cudaGetLastError() == cudaSuccess ? DG_OK : DG_ECUDA;
+  return launch_pdl(mlp_reduce_adam_kernel, (npar + 1 + 31) / 32, 256, 0, st, workspace, nb, npar, (float*)NULL, params,
+                    m, v, step, lr, 0.9f, 0.999f, 1e-8f, loss) == cudaSuccess
+             ? DG_OK
+             : DG_ECUDA;
 }
 
 dg_status dg_mlp_forward(const float* params, int n_out, const float* X, float* y, int64_t n, int tensor_cores,

@@ -62,3 +62,34 @@ def test_overlapped_launches_change_nothing(dg, precision, kind, dim, N, shape, 
         assert np.all(np.isfinite(got[0][1]))
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("batch,n_out,own_stream", [(1, 1, False), (200, 10, True), (4096, 10, False), (5000, 1, True)])
+def test_overlapped_training_changes_nothing(dg, batch, n_out, own_stream):
+    """Training iterations (two gathers into buffers that the last iteration read, gradient, Adam) with a
+    synchronisation after each call and without any."""
+    import torch
+    g = torch.Generator().manual_seed(3)
+    X = torch.randn((20000, 7), generator=g).cuda()
+    Y = torch.randn((20000, n_out), generator=g).cuda()
+    idx = torch.randint(0, 20000, (30, batch), generator=g).cuda()
+    P0 = (0.3 * torch.randn((dg.dg_mlp_nparams(n_out),), generator=g)).cuda()
+    stream = torch.cuda.Stream() if own_stream else None
+    raw = stream.cuda_stream if own_stream else None
+    got = []
+    for apart in (True, False, False):
+        P, m, v = P0.clone(), torch.zeros_like(P0), torch.zeros_like(P0)
+        loss = torch.zeros((1,), dtype=torch.float64, device="cuda")
+        ws = torch.empty((dg.dg_mlp_workspace_bytes(batch, n_out) // 4,), device="cuda")
+        xb, yb = torch.empty((batch, 7), device="cuda"), torch.empty((batch, n_out), device="cuda")
+        torch.cuda.synchronize()
+        wait = torch.cuda.synchronize if apart else (lambda: None)
+        for k in range(30):
+            dg.dg_gather_rows(X, idx[k], xb, raw), wait()
+            dg.dg_gather_rows(Y, idx[k], yb, raw), wait()
+            dg.dg_mlp_train_step(P, m, v, xb, yb if n_out > 1 else yb.reshape(-1), k + 1, 1e-3, loss, ws, raw), wait()
+        torch.cuda.synchronize()
+        got.append((P, m, v, loss))
+    for other in got[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(got[0], other))
+    assert torch.isfinite(got[0][0]).all() and not torch.equal(got[0][0], P0)
