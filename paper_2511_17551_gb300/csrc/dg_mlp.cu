@@ -311,8 +311,9 @@ __device__ __forceinline__ void tile_2x4(const float* a0, const float* a1, const
 // its transpose, its gradient) are 2 x 4 and 4 x 4 register tiles over 256 threads with 16-byte
 // shared-memory reads; the gradient sums stay in registers over the tiles.  With 64 threads, one
 // per unit, and every operand read 4 bytes at a time, a fitting iteration (two
-// gathers, this, Adam) with a batch of 4,096 and ten outputs took 88 us, then 36, and 25 since the launches overlap (dg_launch.cuh); what is left is the
-// chain of eight barriers of one tile per CTA (128 CTAs) and the launches.
+// gathers, this, Adam) with a batch of 4,096 and ten outputs took 88 us, then 36, and 25 since the
+// launches overlap (dg_launch.cuh); what is left is the chain of eight barriers of one tile per CTA
+// (128 CTAs) and the launches.
 __global__ void __launch_bounds__(TT) mlp_grad_kernel(const float* P, int no, const float* X, const float* t, int B,
                                                       float* partial) {
   extern __shared__ __align__(16) unsigned char raw[];
