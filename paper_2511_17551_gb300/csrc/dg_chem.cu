@@ -214,11 +214,14 @@ struct ChemRow32 {
   float nf[NSPEC], dn[NSPEC], jf[NSPEC], jb[NSPEC];
   // bits s, 5 + s, 10 + s, 15 + s: these are not zero; bit 20: third body
   int mask;
+  // bits s: nu''_s > 0; 5 + s, 10 + s: nu'_s, nu''_s odd; 15 + s, 20 + s: nu'_s, nu''_s one
+  int mask2;
   double dn64[NSPEC];
 };
 struct ChemTab32 {
   dgdd::dd cw[NSPEC], ow[NSPEC];     // 1e-6 / W; 1e6 W 2^-60
   ChemRow32 row[MAXR];
+  int n;                             // rows; reactions switched off (A = 0) are left out
 };
 static_assert(sizeof(ChemTab32) < 16 * 1024, "a kernel argument");
 
@@ -238,19 +241,39 @@ static_assert(sizeof(ChemTab32) < 16 * 1024, "a kernel argument");
 // pairs are integer work (as instructions they took a quarter of the FP64 pipe's time).  All of it in
 // pairs, logarithms, g and delta too, missed the FP64 source by a tenfold larger maximum near
 // equilibrium.
-// Returns false where the pairs do not hold (a concentration that is not between 1e-24 and
-// 1e6 mol/cm^3, zero and negative ones among them, or a result that is not finite); the caller
-// then evaluates the node in FP64.
+//
+// GEN = false holds where every concentration lies between 1e-24 and 1e6 mol/cm^3.  GEN = true takes
+// absent species (c = 0), negative ones (overshoots next to a front) and concentrations down to
+// 9e-43 mol/cm^3 as well: ln |c_s| (of 2^60 |c_s| where |c_s| < 1e-24), 0 for an absent species, so that
+// the exponentials give the products without it; a direction that consumes an absent species has
+// rate zero, a negative species gives its sign by the parity of nu, and for both the derivative
+// is the explicit product without c_s for nu = 1 and zero for higher powers, as in chem_node.  For
+// other species the values are those of GEN = false.
+// Returns false where the pairs do not hold (other concentrations, or a result that is not
+// finite).
+template <bool GEN>
 __device__ __forceinline__ bool chem_node_dd(const float* uu, int np, double Td, const ChemTab32& t,
-                                             const dgdd::dd* exp2, const double* sp, int nr, dgdd::dd* om,
-                                             dgdd::dd* jpi) {
+                                             const dgdd::dd* exp2, const double* sp, dgdd::dd* om, dgdd::dd* jpi) {
   using namespace dgdd;
+  constexpr float UP = 1152921504606846976.0f;  // 2^60
   dd c[NSPEC], lc[NSPEC], jd[NSPEC], j1[NSPEC];
   double w[NSPEC];
+  int none = 0, minus = 0, tiny = 0;  // GEN: bit s of an absent, a negative, a scaled species
   bool ok = true;
 #pragma unroll
   for (int s = 0; s < NSPEC; ++s) {
-    c[s] = mul(t.cw[s], uu[s * np]);
+    const float us = uu[s * np];
+    c[s] = mul(t.cw[s], GEN ? fabsf(us) : us);
+    if (GEN) {
+      if (us < 0.f) minus |= 1 << s;
+      if (us == 0.f) {
+        none |= 1 << s;
+        c[s] = make(1.f, 0.f);
+      } else if (c[s].h < 1e-24f) {
+        tiny |= 1 << s;
+        c[s] = mul(make(t.cw[s].h * UP, t.cw[s].l * UP), fabsf(us));
+      }
+    }
     ok = ok && c[s].h >= 1e-24f && c[s].h <= 1e6f;
   }
   if (!ok) return false;
@@ -262,11 +285,16 @@ __device__ __forceinline__ bool chem_node_dd(const float* uu, int np, double Td,
     const double* q = sp + SP_W * s;
     double l;
     lc[s] = log_(c[s], exp2, &l);
+    if (GEN && (tiny >> s & 1)) {
+      constexpr double ln_up = 60.0 * 0.69314718055994530942;
+      lc[s] = add(lc[s], make(-(float)ln_up, -(float)(ln_up - (double)(float)ln_up)));
+      l -= ln_up;
+    }
     w[s] = (q[2] + Td * (q[3] + Td * (q[4] + Td * (q[5] + Td * q[6]))) + q[7] * iTd - q[8] * lnTd) + l + mlnP;
     om[s] = jd[s] = j1[s] = make(0.f, 0.f);
   }
 #pragma unroll 1
-  for (int r = 0; r < nr; ++r) {
+  for (int r = 0; r < t.n; ++r) {
     const ChemRow32& row = t.row[r];
     const int mask = row.mask;  // the same for every node: no divergence below
     double dl = 0.0;
@@ -281,17 +309,35 @@ __device__ __forceinline__ bool chem_node_dd(const float* uu, int np, double Td,
       if (mask & (1 << s)) acc_mul(tf, lc[s], row.nf[s]);
     const dd delta = from_double(dl);
     tf = norm(tf);
-    const dd pf = exp_scaled(tf, SCALE2, exp2);
+    dd pf = exp_scaled(tf, SCALE2, exp2);
     dd pb = exp_scaled(add(tf, delta), SCALE2, exp2), dp = add(pf, neg(pb));
     if (fabsf(delta.h) < 0.0625f) {
       dp = neg(mul(pf, expm1_small(delta)));
       pb = add(pf, neg(dp));
     }
-    dd Rr = dp, pfM = pf, pbM = pb;
+    // GEN: pf and pb are the products over the species that are there; their signs, 0 where a
+    // species of theirs is absent
+    float sf = 1.f, sb = 1.f;
+    const dd qf = pf, qb = pb;
+    if (GEN) {
+      if (__popc(minus & row.mask2 >> 5) & 1) sf = -1.f;
+      if (__popc(minus & row.mask2 >> 10) & 1) sb = -1.f;
+      pf = none & mask & 31 ? make(0.f, 0.f) : make(sf * qf.h, sf * qf.l);
+      pb = none & row.mask2 & 31 ? make(0.f, 0.f) : make(sb * qb.h, sb * qb.l);
+      if (none & (mask | row.mask2) & 31 || sf != sb || sf < 0.f)
+        dp = none & (mask | row.mask2) & 31 || sf != sb ? add(pf, neg(pb)) : neg(dp);
+    }
+    dd Rr = dp, pfM = pf, pbM = pb, M = make(1.f, 0.f);
     if (mask & (1 << 20)) {
-      dd M = mul(row.eff[0], c[0]);
+      // (GEN: the concentrations themselves; adding a zero changes nothing)
+      auto conc = [&](int s) {
+        if (!GEN) return c[s];
+        const float f = none >> s & 1 ? 0.f : (minus >> s & 1 ? -1.f : 1.f) * (tiny >> s & 1 ? 1.f / UP : 1.f);
+        return make(f * c[s].h, f * c[s].l);
+      };
+      M = mul(row.eff[0], conc(0));
 #pragma unroll
-      for (int s = 1; s < NSPEC; ++s) acc_mul(M, row.eff[s], c[s]);
+      for (int s = 1; s < NSPEC; ++s) acc_mul(M, row.eff[s], conc(s));
       M = norm(M);
       Rr = mul(dp, M);
       pfM = mul(pf, M);
@@ -308,12 +354,37 @@ __device__ __forceinline__ bool chem_node_dd(const float* uu, int np, double Td,
       if (mask & (1 << (10 + s))) acc_mul(j1[s], pfM, row.jf[s]);
       if (mask & (1 << (15 + s))) acc_mul(j1[s], pbM, row.jb[s]);
     }
+    if (GEN) {  // absent and negative species: the explicit products (j1 is not used for them)
+#pragma unroll
+      for (int s = 0; s < NSPEC; ++s) {
+        const int b = 1 << s;
+        if (!((none | minus) & mask >> 5 & b)) continue;
+        dd e = make(0.f, 0.f);
+        const float up = tiny & b ? -UP : -1.f;  // 1 / c_s = up / |scaled c_s|
+        if (row.mask2 >> 15 & b && !(none & mask & 31 & ~b)) {
+          const dd q = none & b ? make(sf * qf.h, sf * qf.l) : div(pf, c[s]);
+          e = none & b ? q : make(up * q.h, up * q.l);
+        }
+        if (row.mask2 >> 20 & b && !(none & row.mask2 & 31 & ~b)) {
+          const dd q = none & b ? make(sb * qb.h, sb * qb.l) : div(pb, c[s]);
+          e = add(e, none & b ? neg(q) : make(-up * q.h, -up * q.l));
+        }
+        acc_mul(jd[s], mul(e, M), row.dn[s]);
+      }
+    }
   }
   const float down = bits((uint32_t)(127 - SCALE2) << 23);
 #pragma unroll
   for (int s = 0; s < NSPEC; ++s) {
     om[s] = mul(norm(om[s]), t.ow[s]);
-    const dd j = add(norm(jd[s]), div(norm(j1[s]), c[s]));
+    dd j = norm(jd[s]);
+    if (!GEN) {
+      j = add(j, div(norm(j1[s]), c[s]));
+    } else if (!((none | minus) >> s & 1)) {
+      const dd q = div(norm(j1[s]), c[s]);
+      const float up = tiny >> s & 1 ? UP : 1.f;
+      j = add(j, make(up * q.h, up * q.l));
+    }
     ok = ok && isfinite(om[s].h) && isfinite(j.h);
     jpi[s] = j.h < 0.f ? make(fmul(-j.h, down), fmul(-j.l, down)) : make(0.f, 0.f);
   }
@@ -326,10 +397,19 @@ __device__ __noinline__ void chem_node_rare(const float* uu, int np, double Tk, 
   double o[NSPEC], j[NSPEC];
   chem_node<float>(uu, np, Tk, sp, reac, nr, o, j);
 #pragma unroll
-  for (int s = 0; s < NSPEC; ++s) {
-    om[s] = dgdd::from_double(o[s]);
-    jpi[s] = dgdd::from_double(j[s]);
+  for (int s = 0; s < NSPEC; ++s) {  // (subnormals kept)
+    split_f64(o[s], om[s].h, om[s].l);
+    split_f64(j[s], jpi[s].h, jpi[s].l);
   }
+}
+
+// a node outside the usual range of concentrations.  A function of its own, so that the kernels keep
+// the registers of the usual case.  576,000 nodes, one of five species absent everywhere: 346 us (all
+// present: 237; every node in FP64: 1,274); absent in every second node, so that a warp runs both, 640.
+__device__ __noinline__ void chem_node_general(const float* uu, int np, double Tk, const ChemTab32& t,
+                                               const dgdd::dd* exp2, const double* sp, const double* reac, int nr,
+                                               dgdd::dd* om, dgdd::dd* jpi) {
+  if (!chem_node_dd<true>(uu, np, Tk, t, exp2, sp, om, jpi)) chem_node_rare(uu, np, Tk, sp, reac, nr, om, jpi);
 }
 
 // The plain source of one node in the two forms: the rates in the form's arithmetic, and
@@ -356,9 +436,9 @@ struct Chem32 {  // mixed form
   }
   __device__ __forceinline__ void rates(const float* uu, int np, double Tk, const Tab& e, const ChemTab32& t,
                                         const double* sp, const double* reac, int nr) {
-    if (!chem_node_dd(uu, np, Tk, t, e.exp2, sp, nr, om, jpi)) {
+    if (!chem_node_dd<false>(uu, np, Tk, t, e.exp2, sp, om, jpi)) {
       dgdd::dd o[NSPEC], j[NSPEC];
-      chem_node_rare(uu, np, Tk, sp, reac, nr, o, j);
+      chem_node_general(uu, np, Tk, t, e.exp2, sp, reac, nr, o, j);
 #pragma unroll
       for (int s = 0; s < NSPEC; ++s) {
         om[s] = o[s];
@@ -910,7 +990,8 @@ cudaError_t dg_chem_init(DgThermo* th, const double* species_host, const double*
   }
   for (int r = 0; r < nr; ++r) {
     const double* o = rows + RX_W * r;
-    ChemRow32& w = t32->row[r];
+    if (reac_host[19 * r + 16] == 0.0) continue;  // ln A has no pair, and both rates are zero
+    ChemRow32& w = t32->row[t32->n++];
     w.lnA = dgdd::from_double(o[16]);
     w.beta = dgdd::from_double(o[17]);
     w.mtheta = dgdd::from_double(-o[18]);
@@ -924,6 +1005,8 @@ cudaError_t dg_chem_init(DgThermo* th, const double* species_host, const double*
       w.jb[s] = -b * (b - a);
       w.mask |= (w.nf[s] != 0.f) << s | (w.dn[s] != 0.f) << (5 + s) | (w.jf[s] != 0.f) << (10 + s) |
                 (w.jb[s] != 0.f) << (15 + s);
+      const int ia = (int)a, ib = (int)b;
+      w.mask2 |= (ib > 0) << s | (ia & 1) << (5 + s) | (ib & 1) << (10 + s) | (ia == 1) << (15 + s) | (ib == 1) << (20 + s);
     }
     if (o[10] != 0.0) w.mask |= 1 << 20;
   }
