@@ -417,15 +417,17 @@ __device__ __noinline__ void chem_node_general(const float* uu, int np, double T
 // source goes through these, so that they agree bit for bit.
 struct Chem64 {  // FP64 form
   struct Tab {};
+  struct Args {};  // the pairs' table is no argument of this form's kernels
   double om[NSPEC], jpi[NSPEC];
   __device__ __forceinline__ static void stage(Tab&, const dgdd::dd*) {}
-  __device__ __forceinline__ void rates(const double* uu, int np, double Tk, const Tab&, const ChemTab32&,
+  __device__ __forceinline__ void rates(const double* uu, int np, double Tk, const Tab&, const Args&,
                                         const double* sp, const double* reac, int nr) {
     chem_node<double>(uu, np, Tk, sp, reac, nr, om, jpi);
   }
   __device__ __forceinline__ double source(int s, double dt) const { return om[s] / (1.0 + dt * jpi[s]); }
 };
 struct Chem32 {  // mixed form
+  typedef ChemTab32 Args;
   struct Tab {
     dgdd::dd exp2[dgdd::EXP_TAB];  // 2^(j/128), in shared memory
   };
@@ -454,13 +456,17 @@ struct Chem32 {  // mixed form
 template <typename T> struct ChemForm;
 template <> struct ChemForm<double> { typedef Chem64 type; typedef double step; };
 template <> struct ChemForm<float> { typedef Chem32 type; typedef dgdd::dd step; };
+template <typename T> using ChemArgs = typename ChemForm<T>::type::Args;
+// (Launch bounds of the kernels below: the FP64 instances are held to 168 registers, three CTAs of 128 on
+// an SM; unbounded they took 178 to 186 and two: plain 1,255 -> 1,247 us at 576,000 nodes, refreshes
+// 1,309 -> 1,280.)
 __device__ __forceinline__ void form_step(double dt, double& out) { out = dt; }
 __device__ __forceinline__ void form_step(double dt, dgdd::dd& out) { out = dgdd::from_double(dt); }
 
 template <typename T>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 1)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 3)
 chem_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, const double* sp_raw, const double* reac,
-            int nr, const __grid_constant__ ChemTab32 tab, const dgdd::dd* exp2, const double* dtp, T* src) {
+            int nr, const __grid_constant__ ChemArgs<T> tab, const dgdd::dd* exp2, const double* dtp, T* src) {
   typedef typename ChemForm<T>::type Form;
   __shared__ typename Form::Tab t;
   Form::stage(t, exp2);
@@ -581,11 +587,13 @@ __device__ __forceinline__ int64_t sampled_node(int64_t t, int64_t total, uint64
 // The first `checks` CTAs of the grid evaluate the plain source at every tile's sampled node
 // instead (one thread per tile, S into `sampled`) for the next kernel to compare with: a chain
 // of one evaluation that fills a fraction of the GPU (28 us as a kernel of its own at 18,000
-// tiles) runs beside the network.
+// tiles) runs beside the network.  In the FP64 form there are none (checks = 0): both sides need the
+// FP64 pipe, so nothing is hidden, and tiles that the other tests reject would be evaluated too (18,000
+// tiles: all accepted 235 against 220 us, all rejected 1,439 against 1,368).
 template <typename T>
 __global__ void __launch_bounds__(dgtc5::THREADS, sizeof(T) == 4 ? 5 : 3)
 chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, const double* sp_raw,
-                    const double* reac, int nr, const __grid_constant__ ChemTab32 tab, const dgdd::dd* exp2,
+                    const double* reac, int nr, const __grid_constant__ ChemArgs<T> tab, const dgdd::dd* exp2,
                     const DgChemMlp* mlp, const double* dtp, T* src, unsigned char* flags, float* corr,
                     const unsigned char* trust, int cmode, int checks, T* sampled, uint64_t call,
                     unsigned long long* stats) {
@@ -598,7 +606,7 @@ chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, co
     pdl_wait();
     if (cmode != 2 && blockIdx.x == 0 && threadIdx.x == 0) stats[2] = 0;  // chem_fallback_kernel's tile counter
   };
-  if ((int)blockIdx.x < checks) {
+  if (sizeof(T) == 4 && (int)blockIdx.x < checks) {
     typename Form::Tab& tb = *reinterpret_cast<typename Form::Tab*>(smem_raw);
     Form::stage(tb, exp2);
     enter();
@@ -718,15 +726,36 @@ chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, co
   dgtc5::run_tiles<10, CHEM_NR>(s, total, prod, cons, skip, checks);
 }
 
+// the FP64 form's check evaluations: the plain source at the sampled node of each tile that is
+// still accepted, one thread per tile
+__global__ void __launch_bounds__(128, 3)
+chem_sampled_kernel(const double* u, const double* Tc, int64_t K, int np, int dim, const double* sp_raw,
+                    const double* reac, int nr, const double* dtp, const unsigned char* flags, double* sampled,
+                    uint64_t call) {
+  pdl_wait();
+  const int nv = NSPEC + dim + 1;
+  const int64_t total = K * np, t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t * 32 >= total || flags[t]) return;
+  int64_t k;
+  int node;
+  const int64_t i = sampled_node(t, total, call);
+  split_node(i, np, k, node);
+  Chem64 f;
+  f.rates(u + k * nv * np + node, np, Tc[i], Chem64::Tab(), Chem64::Args(), sp_raw, reac, nr);
+  const double dt = dtp ? *dtp : 0.0;
+#pragma unroll
+  for (int s = 0; s < NSPEC; ++s) sampled[NSPEC * t + s] = f.source(s, dt);
+}
+
 // a warp at a time takes the next tile (stats[2] counts them, set to zero by chem_mlp_tc5_kernel):
 // the sampled check if it is still accepted (the learned source at the sampled node against the
-// plain one that chem_mlp_tc5_kernel left), then, if rejected, the plain source at its nodes;
+// plain one in `sampled`), then, if rejected, the plain source at its nodes;
 // counts nodes.  Rejected tiles cluster where the rates are large; with a fixed share of the tiles
 // per warp a learned evaluation takes 5 % longer (18,000 tiles, 44 % rejected).
 template <typename T>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 1)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 3)
 chem_fallback_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, const double* sp_raw,
-                     const double* reac, int nr, const __grid_constant__ ChemTab32 tab, const dgdd::dd* exp2,
+                     const double* reac, int nr, const __grid_constant__ ChemArgs<T> tab, const dgdd::dd* exp2,
                      const DgChemMlp* mlp, const double* dtp, T* src, unsigned char* flags, const T* sampled,
                      uint64_t call, unsigned long long* stats) {
   typedef typename ChemForm<T>::type Form;
@@ -855,9 +884,9 @@ __device__ __forceinline__ bool refresh_node(const Chem32& p, dgdd::dd dt, doubl
 }
 
 template <typename T>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 1)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 3)
 chem_refresh_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, const double* sp_raw,
-                    const double* reac, int nr, const __grid_constant__ ChemTab32 tab, const dgdd::dd* exp2,
+                    const double* reac, int nr, const __grid_constant__ ChemArgs<T> tab, const dgdd::dd* exp2,
                     const DgChemMlp* mlp, const double* dtp, T* src, float* corr, unsigned char* flags,
                     unsigned char* trust) {
   typedef typename ChemForm<T>::type Form;
@@ -1028,7 +1057,7 @@ template <typename T>
 static cudaError_t chem_learned(DgThermo* th, const T* u, const double* dt_dev, int refresh, cudaStream_t s) {
   const int64_t total = th->K * th->np, ntiles = (total + 31) / 32;
   const DgChemMlp* m = (const DgChemMlp*)th->chem_mlp;
-  const ChemTab32& tab = *(const ChemTab32*)th->chem_tab32;
+  const ChemArgs<T>& tab = *(const ChemArgs<T>*)th->chem_tab32;  // (the FP64 form's is empty)
   const dgdd::dd* e2 = (const dgdd::dd*)th->chem_exp2;
   const size_t smem = sizeof(dgtc5::Smem<10, CHEM_NR>);
   auto k1 = chem_mlp_tc5_kernel<T>;
@@ -1050,12 +1079,18 @@ static cudaError_t chem_learned(DgThermo* th, const T* u, const double* dt_dev, 
     return e;
   }
   const int cmode = th->chem_corr && th->chem_trust && th->corr_valid ? 1 : 0;
-  const unsigned checks = (unsigned)((ntiles + dgtc5::THREADS - 1) / dgtc5::THREADS);
+  const unsigned per_tile = (unsigned)((ntiles + 127) / 128), checks = sizeof(T) == 4 ? per_tile : 0;
+  static_assert(dgtc5::THREADS == 128, "one thread per tile");
   const uint64_t call = th->chem_calls++;
   e = launch_pdl(k1, checks + g1, dgtc5::THREADS, smem, s, u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac,
                  th->nr, tab, e2, m, dt_dev, (T*)th->src, th->chem_flags, th->chem_corr, th->chem_trust, cmode,
                  (int)checks, (T*)th->chem_sampled, call, th->chem_stats);
   if (e != cudaSuccess) return e;
+  if constexpr (sizeof(T) == 8) {
+    e = launch_pdl(chem_sampled_kernel, per_tile, 128, 0, s, u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac,
+                   th->nr, dt_dev, th->chem_flags, (double*)th->chem_sampled, call);
+    if (e != cudaSuccess) return e;
+  }
   int64_t g3 = (ntiles + 3) / 4;
   if (g3 > 152 * 5) g3 = 152 * 5;
   return launch_pdl(chem_fallback_kernel<T>, (unsigned)g3, 128, 0, s, u, th->T, th->K, th->np, th->dim, th->species_raw,
@@ -1069,13 +1104,12 @@ cudaError_t dg_chem_source(DgThermo* th, const void* u, int f32, const double* d
     return f32 ? chem_learned<float>(th, (const float*)u, dt_dev, refresh, s)
                : chem_learned<double>(th, (const double*)u, dt_dev, refresh, s);
   const unsigned grid = grid_of(th->K * th->np);
-  const ChemTab32& tab = *(const ChemTab32*)th->chem_tab32;
   const dgdd::dd* e2 = (const dgdd::dd*)th->chem_exp2;
   if (f32)
     return launch_pdl(chem_kernel<float>, grid, 128, 0, s, (const float*)u, th->T, th->K, th->np, th->dim, th->species_raw,
-                      th->reac, th->nr, tab, e2, dt_dev, (float*)th->src);
+                      th->reac, th->nr, *(const ChemTab32*)th->chem_tab32, e2, dt_dev, (float*)th->src);
   return launch_pdl(chem_kernel<double>, grid, 128, 0, s, (const double*)u, th->T, th->K, th->np, th->dim,
-                    th->species_raw, th->reac, th->nr, tab, e2, dt_dev, (double*)th->src);
+                    th->species_raw, th->reac, th->nr, Chem64::Args(), e2, dt_dev, (double*)th->src);
 }
 
 cudaError_t dg_chem_mlp_set(DgThermo* th, const float* params_host, const double* st) {

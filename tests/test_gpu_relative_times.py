@@ -1,0 +1,59 @@
+"""Times of calls against other calls on the same GPU, where a change once made one of them slower:
+each bound lies between the two ratios measured, which its test states."""
+import numpy as np
+import pytest
+
+import cases
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dg():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2511_17551_gb300 as dg
+    dg.lib()
+    return dg
+
+
+def _chem_ms(dg, s, u, r, n=10):
+    for _ in range(2):
+        dg.dg_rhs(s.ctx, u, r)
+    dg.dg_profile(s.ctx, 1)
+    dg.dg_profile_read(s.ctx)
+    for _ in range(n):
+        dg.dg_rhs(s.ctx, u, r)
+    p = dg.dg_profile_read(s.ctx)
+    dg.dg_profile(s.ctx, 0)
+    return p["chem"][0] / n
+
+
+def test_fp64_learned_source_with_every_tile_rejected(dg):
+    """FP64 form: network, tests and fallback cost 1.10 plain evaluations where every tile leaves the
+    training box; with check evaluations for rejected tiles too they cost 1.15."""
+    import torch
+    x, _ = dg.dg_lgl_nodes(4)
+    xyz, nbr, face = W.ogrid_mesh(x, 24, 24, 8)
+    w = W.mixture_primitive(xyz, rho=0.1, vel=(2400.0, 0.0, 0.0), T=300.0, seed=7, cylinder=0.5, hot=(1.2, 3000.0))
+    kinds, bcp = cases.mixture_bc(w)
+    s = dg.Solver(3, 4, xyz, nbr, face, n_species=5, species=W.species_table(), volume_flux=1, bc_kind=kinds, bc_prim=bcp,
+                  reactions=W.reaction_table())
+    try:
+        s.set_primitive(w)
+        u = torch.from_numpy(s.get_state()[0]).cuda()
+        r = torch.empty_like(u)
+        plain = _chem_ms(dg, s, u, r)
+        p = (0.3 * np.random.default_rng(3).normal(size=dg.dg_mlp_nparams(10))).astype(np.float32)
+        st = np.zeros(53)
+        st[7:14], st[24:34], st[34], st[35] = 1.0, 1.0, 1e2, 1e3
+        st[36:43], st[43:50], st[50:52] = 1e30, -1e30, 1e30
+        dg.dg_set_surrogate(s.ctx, p, st, which=dg.DG_SURROGATE_SOURCE)  # an empty trust box
+        learned = _chem_ms(dg, s, u, r)
+        assert dg.dg_surrogate_stats(s.ctx, dg.DG_SURROGATE_SOURCE)[0] == 0
+        print("plain, all rejected", plain, learned, learned / plain)
+        assert learned < 1.12 * plain, (plain, learned)
+    finally:
+        s.close()
