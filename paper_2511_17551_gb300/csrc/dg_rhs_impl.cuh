@@ -1268,9 +1268,13 @@ __global__ void __launch_bounds__(128) positivity_kernel(const DgArgs a, real* u
   constexpr int EPW = NP >= 128 ? 1 : 128 / NP;
   static_assert(EPW <= 32, "flag mask");
   pdl_wait();
-  trigger();
   const int lane = threadIdx.x & 31;
   const int64_t k0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * EPW;
+  // The next kernel's CTAs: behind the screening, since resident early they leave the right-hand side
+  // after them unevenly placed (N = 2, 20^3 elements with indicator and limiter, four steps: 749 against 1,163 us;
+  // 14^3, N = 3: 585 against 672); at once where the grid leaves most SMs free (10^3, N = 2: 546 against 564)
+  const bool early = gridDim.x <= 64;
+  if (early) trigger();
   if (k0 >= a.K) return;  // uniform per warp
   const int ch = (int)((a.K - k0) < EPW ? (a.K - k0) : EPW) * NP;
   const real tol = sizeof(real) == 4 ? real(1e-6) : real(1e-14);
@@ -1310,6 +1314,7 @@ __global__ void __launch_bounds__(128) positivity_kernel(const DgArgs a, real* u
     if (!ok) flag |= 1u << el;
   }
   flag = __reduce_or_sync(0xffffffffu, flag);
+  if (!early) trigger();
   while (flag) {
     const int el = __ffs(flag) - 1;
     flag &= flag - 1;
@@ -1726,7 +1731,10 @@ __global__ void __launch_bounds__(IndShape<DIM, N>::THREADS) indicator_kernel(co
   constexpr int NP = S::NP, N1 = S::N1, NV = NSP + DIM + 1, ROW = I::ROW;
   __shared__ real sf[I::EPC * ROW];
   pdl_wait();
-  trigger();
+  // (27-node elements: behind the transforms, 34^3 elements, four steps 2,115 -> 1,930 us; the others lose
+  // up to 5 % on small meshes by that)
+  constexpr bool early = !(DIM == 3 && N == 2);
+  if (early) trigger();
   const BasisTab<real>& B = c_tab[N];
   const int tid = threadIdx.x;
   const int64_t e0 = (int64_t)blockIdx.x * I::EPC;
@@ -1776,6 +1784,7 @@ __global__ void __launch_bounds__(IndShape<DIM, N>::THREADS) indicator_kernel(co
     }
     if (I::WARP) __syncwarp();
   }
+  if (!early) trigger();
   real Et = 0, E1 = 0, Eh1 = 0, Eh2 = 0;
 #pragma unroll 4
   for (int node = lane; node < NP; node += step) {
