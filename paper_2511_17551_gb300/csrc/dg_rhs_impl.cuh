@@ -96,15 +96,20 @@ struct Swizzle {
 //   3D one gas, N = 4: 160 threads (2 elements, 150 lines), 4 CTAs: 196 -> 162 us at 26^3 elements (96
 //     threads hold 75 lines, and at 8 CTAs spilled 128 bytes); Euler 134 -> 109, FP64 986 -> 831 (16^3)
 //   N = 7 without viscous terms: 2 CTAs, 161 -> 114 us (14^3; at 3 it spilled 548 bytes)
-//   2D: 128 threads (16 elements at N = 3), 7 CTAs, 96.3 -> 92.2 us (512 x 256)
+//   2D: 128 threads (16 elements at N = 3), 7 CTAs, 96.3 -> 92.2 us (512 x 256).  The other flux pairs (at
+//     most 5 CTAs, launch_ctas) are then held to 96 registers: at N = 7 that spilled 264 bytes, so they
+//     keep 96 threads and 128 registers there (Kennedy-Gruber, 80^2 elements, four steps 994 -> 797 us)
 //   mixtures: 96 threads, 5 CTAs at N = 3 (131 -> 113 us, 28^3) and 4 at N = 4 (180 -> 171, 24^3) instead of
 //     192 threads and 3 CTAs; FP64 keeps 192 (300 against 337 us at 12^3)
 //   FP64 one gas: the FP64 pipe needs few warps, 4 CTAs (2D: 5) instead of 7 or 8 shed 700 to 1,700 bytes of
 //     spills: N = 3 Euler 1038 -> 996 us (24^3), N = 2 550 -> 521, 2D N = 3 529 -> 507
-template <int DIM, int N, int NSP>
+template <int DIM, int N, int NSP, bool PROD>
 struct CtaShape {
   static constexpr bool F64 = sizeof(real) == 8;
-  static constexpr int TPB = NSP > 1 ? (F64 ? 192 : 96) : DIM == 2 ? (F64 ? 96 : 128) : N == 4 ? 160 : 96;
+  static constexpr int TPB = NSP > 1    ? (F64 ? 192 : 96)
+                             : DIM == 2 ? (F64 || (N == 7 && !PROD) ? 96 : 128)
+                             : N == 4   ? 160
+                                        : 96;
   static constexpr int CAP = NSP > 1  ? (F64 ? 3 : N == 3 ? 5 : 4)
                              : F64      ? (DIM == 2 ? 5 : 4)
                              : DIM == 2 ? 7
@@ -112,12 +117,12 @@ struct CtaShape {
                              : N == 7   ? 2
                                         : 8;
 };
-template <int DIM, int N, int NSP, bool NS, bool AL = true>
+template <int DIM, int N, int NSP, bool NS, bool AL>
 struct Layout {
   using S = Shape<DIM, N>;
   static constexpr int NV = NSP + DIM + 1;
   static constexpr int NP = S::NP;
-  static constexpr int EPB = epb<DIM, N, CtaShape<DIM, N, NSP>::TPB>();
+  static constexpr int EPB = epb<DIM, N, CtaShape<DIM, N, NSP, AL>::TPB>();
   static constexpr int NQ = DIM + 3;                // rho, v, p, beta(=rho/p)
   static constexpr int NFV = NS ? DIM * (DIM + 1) : 0;
   static constexpr int FACE_NODES = 2 * DIM * S::LPD;  // per element
@@ -154,7 +159,7 @@ struct Layout {
   static constexpr int PC = FV + EPB * SFV;          // mixtures: p, c per node
   static constexpr int DU = PC + EPB * SPC;           // prefetched RK register du
   // resident-CTA target, lowered where shared memory binds
-  static constexpr int CAP = CtaShape<DIM, N, NSP>::CAP;
+  static constexpr int CAP = CtaShape<DIM, N, NSP, AL>::CAP;
   static constexpr int ctas_of(size_t bytes) {
     return (int)((227 * 1024) / (bytes + 1024)) >= CAP ? CAP : (int)((227 * 1024) / (bytes + 1024));
   }
@@ -343,7 +348,7 @@ __device__ __forceinline__ int outer_state(const DgArgs& a, const KConst& kc, in
 
 // ------------------------------------------------------------------ main RHS / RK kernel
 // the runtime-choice kernel (FL = 0) carries more live branches: at most 5 CTAs per SM
-// (up to 136 registers a thread at 96 threads; 3 of the 160-thread CTAs of N = 4) instead of 8, so
+// (up to 128 registers a thread at 96 threads; 3 of the 160-thread CTAs of N = 4) instead of 8, so
 // that it does not spill; the split forms (FL >= 2) hold both nodes' conserved states per flux pair:
 // at most 6 (96 registers; at 7 the allocator is held to 80 and spills)
 template <int DIM, int N, int NSP, bool NS, int FL>
