@@ -117,12 +117,13 @@ struct CtaShape {
                              : N == 7   ? 2
                                         : 8;
 };
-template <int DIM, int N, int NSP, bool NS, bool AL>
+// ONE: one element a CTA
+template <int DIM, int N, int NSP, bool NS, bool AL, bool ONE = false>
 struct Layout {
   using S = Shape<DIM, N>;
   static constexpr int NV = NSP + DIM + 1;
   static constexpr int NP = S::NP;
-  static constexpr int EPB = epb<DIM, N, CtaShape<DIM, N, NSP, AL>::TPB>();
+  static constexpr int EPB = ONE ? 1 : epb<DIM, N, CtaShape<DIM, N, NSP, AL>::TPB>();
   static constexpr int NQ = DIM + 3;                // rho, v, p, beta(=rho/p)
   static constexpr int NFV = NS ? DIM * (DIM + 1) : 0;
   static constexpr int FACE_NODES = 2 * DIM * S::LPD;  // per element
@@ -351,19 +352,21 @@ __device__ __forceinline__ int outer_state(const DgArgs& a, const KConst& kc, in
 // (up to 128 registers a thread at 96 threads; 3 of the 160-thread CTAs of N = 4) instead of 8, so
 // that it does not spill; the split forms (FL >= 2) hold both nodes' conserved states per flux pair:
 // at most 6 (96 registers; at 7 the allocator is held to 80 and spills)
-template <int DIM, int N, int NSP, bool NS, int FL>
+template <int DIM, int N, int NSP, bool NS, int FL, bool ONE>
 constexpr int launch_ctas() {
+  if (ONE) return 1;
   constexpr int most = production_pair<FL> ? 8 : FL ? 6 : (DIM == 3 && N == 4 && NSP == 1) ? 3 : 5;
-  constexpr int minb = Layout<DIM, N, NSP, NS, production_pair<FL>>::MINB;
+  constexpr int minb = Layout<DIM, N, NSP, NS, production_pair<FL>, ONE>::MINB;
   return minb > most ? most : minb;
 }
 // BND = false compiles the kernel for meshes without boundary faces (periodic or closed by
 // connectivity): the interface code then carries no boundary-state branches.
-template <int DIM, int N, int NSP, bool NS, int FL, bool BND = true>
-__global__ void __launch_bounds__(Layout<DIM, N, NSP, NS, production_pair<FL>>::THREADS, launch_ctas<DIM, N, NSP, NS, FL>())
+template <int DIM, int N, int NSP, bool NS, int FL, bool BND = true, bool ONE = false>
+__global__ void __launch_bounds__(Layout<DIM, N, NSP, NS, production_pair<FL>, ONE>::THREADS,
+                                  launch_ctas<DIM, N, NSP, NS, FL, ONE>())
 rhs_kernel(const DgArgs a, const KConst kc) {
   using S = Shape<DIM, N>;
-  using L = Layout<DIM, N, NSP, NS, production_pair<FL>>;
+  using L = Layout<DIM, N, NSP, NS, production_pair<FL>, ONE>;
   constexpr int NV = L::NV, NP = L::NP, N1 = S::N1, EPB = L::EPB, NQ = L::NQ;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   real* sm = reinterpret_cast<real*>(smem_raw);
@@ -1822,10 +1825,17 @@ cudaError_t set_smem(KernelT k, size_t bytes) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-template <int DIM, int N, int NSP, bool NS, int FL, bool BND>
+template <int DIM, int N, int NSP, bool NS, int FL, bool BND, bool ONE = false>
 cudaError_t launch_rhs_b(const DgArgs& a, cudaStream_t st) {
-  using L = Layout<DIM, N, NSP, NS, production_pair<FL>>;
-  auto k = rhs_kernel<DIM, N, NSP, NS, FL, BND>;
+  // FP64, 3D, N = 4: the FP64 pipe of an SM serves a CTA of two elements (five warps of lines) in 94 us and
+  // one of one element (three warps) in 68 (Euler; Navier-Stokes with its gradients 138 and 111).  So while
+  // there is an SM per element, each element gets one.  From 153 elements on two share a CTA, as the
+  // fewer warps per element count (216 elements: 93 us, with one element a CTA they took 122).  Other
+  // degrees gained at every size by the shapes they have.
+  if constexpr (sizeof(real) == 8 && DIM == 3 && N == 4 && NSP == 1 && !ONE)
+    if (a.K <= 152) return launch_rhs_b<DIM, N, NSP, NS, FL, BND, true>(a, st);
+  using L = Layout<DIM, N, NSP, NS, production_pair<FL>, ONE>;
+  auto k = rhs_kernel<DIM, N, NSP, NS, FL, BND, ONE>;
   cudaError_t err = set_smem(k, L::SMEM);
   if (err != cudaSuccess) return err;
   const int64_t grid = (a.K + L::EPB - 1) / L::EPB;
