@@ -350,7 +350,8 @@ dg_status dg_get_metrics(dg_ctx* ctx, double* Ja, double* invJ, int on_device);
 dg_status dg_get_gradients(dg_ctx* ctx, double* grad);
 
 /* Per-kernel device timing (tracing).  While enabled, every kernel launch of the
- * context is bracketed by CUDA events recorded on the context stream.
+ * context is bracketed by CUDA events recorded on the context stream, and each kernel
+ * starts when the one before it has ended (otherwise their launches overlap).
  * dg_profile_read waits for the stream and returns, per kernel kind, the summed
  * device milliseconds and the number of launches since the last read
  * (kinds: DG_PROF_RHS, DG_PROF_GRAD, DG_PROF_INDICATOR, DG_PROF_LAMBDA,

@@ -517,6 +517,7 @@ DgArgs base_args(dg_ctx* c) {
   a.Ja = f32 ? (const void*)c->Ja32 : (const void*)c->Ja64;
   a.invJ = f32 ? (const void*)c->invJ32 : (const void*)c->invJ64;
   a.own_metrics = 1;
+  a.apart = c->prof;
   a.gradW = c->gradW;
   a.nbr = c->nbr;
   a.bc_kind = c->bc_kind;
@@ -1331,7 +1332,7 @@ dg_status dg_profile(dg_ctx* c, int enable) {
     for (int i = 0; i < c->ev_cap; ++i) CK(cudaEventCreate(&c->ev[i]));
   }
   if (!enable && c->ev) prof_flush(c);
-  c->prof = enable ? 1 : 0;
+  c->prof = c->th.apart = enable ? 1 : 0;
   return DG_OK;
 }
 

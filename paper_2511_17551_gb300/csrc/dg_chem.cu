@@ -1068,11 +1068,11 @@ static cudaError_t chem_learned(DgThermo* th, const T* u, const double* dt_dev, 
   const unsigned g1 = (unsigned)(tiles < 152 * 5 ? tiles : 152 * 5);
   if (refresh) {
     if (!th->chem_corr || !th->chem_trust) return cudaErrorInvalidValue;
-    e = launch_pdl(k1, g1, dgtc5::THREADS, smem, s, u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr,
+    e = launch_pdl(th->apart, k1, g1, dgtc5::THREADS, smem, s, u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac, th->nr,
                    tab, e2, m, dt_dev, (T*)th->src, th->chem_flags, th->chem_corr, th->chem_trust, 2, 0, (T*)NULL, 0,
                    (unsigned long long*)NULL);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(chem_refresh_kernel<T>, grid_of(ntiles * 32), 128, 0, s, u, th->T, th->K, th->np, th->dim,
+    e = launch_pdl(th->apart, chem_refresh_kernel<T>, grid_of(ntiles * 32), 128, 0, s, u, th->T, th->K, th->np, th->dim,
                    th->species_raw, th->reac, th->nr, tab, e2, m, dt_dev, (T*)th->src, th->chem_corr, th->chem_flags,
                    th->chem_trust);
     if (e == cudaSuccess) th->corr_valid = 1;
@@ -1082,18 +1082,18 @@ static cudaError_t chem_learned(DgThermo* th, const T* u, const double* dt_dev, 
   const unsigned per_tile = (unsigned)((ntiles + 127) / 128), checks = sizeof(T) == 4 ? per_tile : 0;
   static_assert(dgtc5::THREADS == 128, "one thread per tile");
   const uint64_t call = th->chem_calls++;
-  e = launch_pdl(k1, checks + g1, dgtc5::THREADS, smem, s, u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac,
+  e = launch_pdl(th->apart, k1, checks + g1, dgtc5::THREADS, smem, s, u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac,
                  th->nr, tab, e2, m, dt_dev, (T*)th->src, th->chem_flags, th->chem_corr, th->chem_trust, cmode,
                  (int)checks, (T*)th->chem_sampled, call, th->chem_stats);
   if (e != cudaSuccess) return e;
   if constexpr (sizeof(T) == 8) {
-    e = launch_pdl(chem_sampled_kernel, per_tile, 128, 0, s, u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac,
+    e = launch_pdl(th->apart, chem_sampled_kernel, per_tile, 128, 0, s, u, th->T, th->K, th->np, th->dim, th->species_raw, th->reac,
                    th->nr, dt_dev, th->chem_flags, (double*)th->chem_sampled, call);
     if (e != cudaSuccess) return e;
   }
   int64_t g3 = (ntiles + 3) / 4;
   if (g3 > 152 * 5) g3 = 152 * 5;
-  return launch_pdl(chem_fallback_kernel<T>, (unsigned)g3, 128, 0, s, u, th->T, th->K, th->np, th->dim, th->species_raw,
+  return launch_pdl(th->apart, chem_fallback_kernel<T>, (unsigned)g3, 128, 0, s, u, th->T, th->K, th->np, th->dim, th->species_raw,
                     th->reac, th->nr, tab, e2, m, dt_dev, (T*)th->src, th->chem_flags, (const T*)th->chem_sampled, call,
                     th->chem_stats);
 }
@@ -1106,9 +1106,9 @@ cudaError_t dg_chem_source(DgThermo* th, const void* u, int f32, const double* d
   const unsigned grid = grid_of(th->K * th->np);
   const dgdd::dd* e2 = (const dgdd::dd*)th->chem_exp2;
   if (f32)
-    return launch_pdl(chem_kernel<float>, grid, 128, 0, s, (const float*)u, th->T, th->K, th->np, th->dim, th->species_raw,
+    return launch_pdl(th->apart, chem_kernel<float>, grid, 128, 0, s, (const float*)u, th->T, th->K, th->np, th->dim, th->species_raw,
                       th->reac, th->nr, *(const ChemTab32*)th->chem_tab32, e2, dt_dev, (float*)th->src);
-  return launch_pdl(chem_kernel<double>, grid, 128, 0, s, (const double*)u, th->T, th->K, th->np, th->dim,
+  return launch_pdl(th->apart, chem_kernel<double>, grid, 128, 0, s, (const double*)u, th->T, th->K, th->np, th->dim,
                     th->species_raw, th->reac, th->nr, Chem64::Args(), e2, dt_dev, (double*)th->src);
 }
 

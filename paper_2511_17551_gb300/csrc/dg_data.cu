@@ -297,7 +297,7 @@ dg_status dg_gather_rows(const float* X, int d, const int64_t* idx, int64_t m, f
   if (!X || !idx || !out || d < 1 || m < 1) return DG_EINVAL;
   int64_t g = (m * d + 255) / 256;
   if (g > 152 * 32) g = 152 * 32;
-  return launch_pdl(gather_rows_kernel, (unsigned)g, 256, 0, (cudaStream_t)stream, X, d, idx, m, out) == cudaSuccess
+  return launch_pdl(false, gather_rows_kernel, (unsigned)g, 256, 0, (cudaStream_t)stream, X, d, idx, m, out) == cudaSuccess
              ? DG_OK
              : DG_ECUDA;
 }

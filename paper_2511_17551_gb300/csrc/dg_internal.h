@@ -41,6 +41,7 @@ struct DgArgs {
   const void* Ja;         // [K][dim][dim][np]
   const void* invJ;       // [K][np]
   int own_metrics;        // Ja and invJ are a context's, written once when it was made
+  int apart;              // kernels start one after the other (per-kernel timing)
   void* gradW;            // [K][dim][dim+1][np] (Navier-Stokes): grad_mode 0 the contravariant
                           // viscous fluxes [d][c] = sum_x Ja^d_x f^v_{x,c}; 1 the gradients [x][c]
   int grad_mode;

@@ -22,8 +22,9 @@
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// apart: an ordinary launch, behind the whole kernel before it (a context whose kernels are being timed)
 template <typename... P, typename... A>
-inline cudaError_t launch_pdl(void (*k)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... a) {
+inline cudaError_t launch_pdl(bool apart, void (*k)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... a) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
@@ -33,6 +34,6 @@ inline cudaError_t launch_pdl(void (*k)(P...), unsigned grid, unsigned block, si
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = apart ? 0 : 1;
   return cudaLaunchKernelEx(&cfg, k, static_cast<P>(a)...);
 }

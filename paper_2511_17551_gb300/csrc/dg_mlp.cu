@@ -691,7 +691,7 @@ static dg_status grad_common(const float* P, int no, const float* X, const float
   if (cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return DG_ECUDA;
-  if (launch_pdl(mlp_grad_kernel, nb, TT, smem, st, P, no, X, t, B, ws) != cudaSuccess) return DG_ECUDA;
+  if (launch_pdl(false, mlp_grad_kernel, nb, TT, smem, st, P, no, X, t, B, ws) != cudaSuccess) return DG_ECUDA;
   *nb_out = nb;
   return DG_OK;
 }
@@ -704,7 +704,7 @@ dg_status dg_mlp_grad(const float* params, int n_out, const float* X, const floa
   if (r != DG_OK) return r;
   if (!grad) return DG_EINVAL;
   const int npar = dg_mlp_np(n_out);
-  return launch_pdl(mlp_reduce_adam_kernel, (npar + 1 + 31) / 32, 256, 0, st, workspace, nb, npar, grad, (float*)NULL,
+  return launch_pdl(false, mlp_reduce_adam_kernel, (npar + 1 + 31) / 32, 256, 0, st, workspace, nb, npar, grad, (float*)NULL,
                     (float*)NULL, (float*)NULL, 0, 0.f, 0.f, 0.f, 0.f, loss) == cudaSuccess
              ? DG_OK
              : DG_ECUDA;
@@ -719,7 +719,7 @@ dg_status dg_mlp_train_step(float* params, int n_out, float* m, float* v, const 
   dg_status r = grad_common(params, n_out, X, t, batch, workspace, ws_bytes, st, &nb);
   if (r != DG_OK) return r;
   const int npar = dg_mlp_np(n_out);
-  return launch_pdl(mlp_reduce_adam_kernel, (npar + 1 + 31) / 32, 256, 0, st, workspace, nb, npar, (float*)NULL, params,
+  return launch_pdl(false, mlp_reduce_adam_kernel, (npar + 1 + 31) / 32, 256, 0, st, workspace, nb, npar, (float*)NULL, params,
                     m, v, step, lr, 0.9f, 0.999f, 1e-8f, loss) == cudaSuccess
              ? DG_OK
              : DG_ECUDA;

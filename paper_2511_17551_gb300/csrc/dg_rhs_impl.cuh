@@ -1839,7 +1839,7 @@ cudaError_t launch_rhs_b(const DgArgs& a, cudaStream_t st) {
   cudaError_t err = set_smem(k, L::SMEM);
   if (err != cudaSuccess) return err;
   const int64_t grid = (a.K + L::EPB - 1) / L::EPB;
-  return launch_pdl(k, (unsigned)grid, L::THREADS, L::SMEM, st, a, make_kconst(a));
+  return launch_pdl(a.apart, k, (unsigned)grid, L::THREADS, L::SMEM, st, a, make_kconst(a));
 }
 
 // the production pair of a one-gas 3D mesh without boundary faces runs the kernel
@@ -1861,10 +1861,10 @@ cudaError_t launch_grad_t(const DgArgs& a, cudaStream_t st) {
   cudaError_t err = set_smem(k, smem);
   if (err != cudaSuccess) return err;
   const int64_t grid = (a.K + L::EPB - 1) / L::EPB;
-  err = launch_pdl(k, (unsigned)grid, L::THREADS, smem, st, a, make_kconst(a));
+  err = launch_pdl(a.apart, k, (unsigned)grid, L::THREADS, smem, st, a, make_kconst(a));
   if (err != cudaSuccess || !a.has_bnd) return err;
   const int64_t nn = a.K * Shape<DIM, N>::NP;
-  return launch_pdl(boundary_lift_kernel<DIM, N, NSP>, (unsigned)((nn + 255) / 256), 256, 0, st, a, make_kconst(a));
+  return launch_pdl(a.apart, boundary_lift_kernel<DIM, N, NSP>, (unsigned)((nn + 255) / 256), 256, 0, st, a, make_kconst(a));
 }
 
 template <int DIM, int N, int NSP>
@@ -1873,14 +1873,14 @@ cudaError_t launch_pos_t(const DgArgs& a, void* u, void* ulo, double eps, unsign
   constexpr int NP = Shape<DIM, N>::NP, EPW = NP >= 128 ? 1 : 128 / NP;
   const int64_t warps = (a.K + EPW - 1) / EPW;
   const int64_t grid = (warps * 32 + 127) / 128;
-  return launch_pdl(positivity_kernel<DIM, N, NSP>, (unsigned)grid, 128, 0, st, a, (real*)u, (real*)ulo, eps, nlim);
+  return launch_pdl(a.apart, positivity_kernel<DIM, N, NSP>, (unsigned)grid, 128, 0, st, a, (real*)u, (real*)ulo, eps, nlim);
 }
 
 template <int DIM, int N, int NSP>
 cudaError_t launch_ind_t(const DgArgs& a, double amax, void* out, cudaStream_t st) {
   using I = IndShape<DIM, N>;
   const int64_t grid = (a.K + I::EPC - 1) / I::EPC;
-  return launch_pdl(indicator_kernel<DIM, N, NSP>, (unsigned)grid, I::THREADS, 0, st, a, make_kconst(a), (real)amax,
+  return launch_pdl(a.apart, indicator_kernel<DIM, N, NSP>, (unsigned)grid, I::THREADS, 0, st, a, make_kconst(a), (real)amax,
                     (real*)out);
 }
 #endif  // DG_GENERIC_ONLY
@@ -1983,16 +1983,16 @@ cudaError_t DG_CAT(DG_PREFIX, _lambda)(const DgArgs& a, int slot, cudaStream_t s
   if (grid > 152 * 16) grid = 152 * 16;
   const DG_PREFIX::KConst kc = DG_PREFIX::make_kconst(a);
   if (a.dim == 3 && a.nsp == 1)
-    return launch_pdl(DG_PREFIX::lambda_kernel<3, 1>, (unsigned)grid, bs, 0, st, a, kc, slot);
+    return launch_pdl(a.apart, DG_PREFIX::lambda_kernel<3, 1>, (unsigned)grid, bs, 0, st, a, kc, slot);
   if (a.dim == 2 && a.nsp == 1)
-    return launch_pdl(DG_PREFIX::lambda_kernel<2, 1>, (unsigned)grid, bs, 0, st, a, kc, slot);
+    return launch_pdl(a.apart, DG_PREFIX::lambda_kernel<2, 1>, (unsigned)grid, bs, 0, st, a, kc, slot);
   if (a.dim == 3 && a.nsp == 5)
-    return launch_pdl(DG_PREFIX::lambda_kernel<3, 5>, (unsigned)grid, bs, 0, st, a, kc, slot);
+    return launch_pdl(a.apart, DG_PREFIX::lambda_kernel<3, 5>, (unsigned)grid, bs, 0, st, a, kc, slot);
   return cudaErrorInvalidValue;
 }
 
 cudaError_t DG_CAT(DG_PREFIX, _step_dt)(const DgArgs& a, int slot, int advance_time, cudaStream_t st) {
-  return launch_pdl(DG_PREFIX::step_dt_kernel, 1, 32, 0, st, a, slot, advance_time);
+  return launch_pdl(a.apart, DG_PREFIX::step_dt_kernel, 1, 32, 0, st, a, slot, advance_time);
 }
 
 #endif  // DG_GENERIC_ONLY

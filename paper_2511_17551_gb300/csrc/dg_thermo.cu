@@ -359,13 +359,13 @@ cudaError_t dg_thermo_update(DgThermo* th, const void* u, int f32, cudaStream_t 
   if (th->mode == 1 && th->mlp) return dg_mlp_thermo_update(th, u, f32, s);
   const unsigned grid = grid_of(th->K * th->np);
   if (!f32)
-    return launch_pdl(thermo_update_kernel, grid, 256, 0, s, (const double*)u, th->K, th->np, th->dim, th->species, th->T,
+    return launch_pdl(th->apart, thermo_update_kernel, grid, 256, 0, s, (const double*)u, th->K, th->np, th->dim, th->species, th->T,
                       (double*)th->pc, th->status);
   if (th->dim == 3 && th->np == 64)
-    return launch_pdl(thermo_mixed_kernel<64, 3>, grid, 256, 0, s, (const float*)u, th->K, th->species, th->coef32, th->T,
+    return launch_pdl(th->apart, thermo_mixed_kernel<64, 3>, grid, 256, 0, s, (const float*)u, th->K, th->species, th->coef32, th->T,
                       (float*)th->pc, th->status);
   if (th->dim == 3 && th->np == 125)
-    return launch_pdl(thermo_mixed_kernel<125, 3>, grid, 256, 0, s, (const float*)u, th->K, th->species, th->coef32, th->T,
+    return launch_pdl(th->apart, thermo_mixed_kernel<125, 3>, grid, 256, 0, s, (const float*)u, th->K, th->species, th->coef32, th->T,
                       (float*)th->pc, th->status);
   return cudaErrorInvalidValue;  // mixtures are 3D with N = 3 or 4
 }

@@ -17,6 +17,7 @@ struct DgThermo {
   double* reac;        // device [nr][20] reaction rows (ln A in slot 16)
   void* chem_tab32;    // host: the same rows as double-FP32 pairs, a kernel argument (dg_chem.cu)
   void* chem_exp2;     // device: 2^(j/128) as pairs
+  int apart;           // kernels start one after the other (per-kernel timing)
   int nr;              // number of reactions, 0 = frozen
   void* src;           // device [K][ns][np] chemistry source (form precision)
   void* mlp;           // temperature surrogate weights (device) or null
