@@ -49,3 +49,34 @@ def test_cfl_steps_with_sutherland(dg, precision, tol, N, shape, where):
         assert abs(t_g / t_o - 1) < (1e-12 if tol is None else 1e-5)
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("N,shape", [(2, (3, 2, 5)), (3, (4, 3, 3)), (4, (3, 2, 3)), (7, (2, 2, 3))])
+def test_production_and_runtime_choice_kernel_agree(dg, precision, N, shape):
+    """Sutherland's law with LLF (the kernel of the production pair) and with HLLC (the runtime-choice kernel) on
+    a flow whose traces agree at every face: both interface fluxes are then the flux of that trace, and
+    the right-hand sides differ by roundings (16 times the oracle's floor)."""
+    import torch
+    kw = dict(W.supersonic_tgv_physics())
+    got = []
+    for sf in (0, 1):
+        p = cases.Pair(lambda x: cases.supersonic_tgv(x, None, warp=0.1, shape=shape), 3, N, precision=precision, equations=1,
+                       surface_flux=sf, **kw)
+        try:
+            u_o = p.orc.prim_to_cons(p.mesh_o[3])
+            if precision:
+                u_o = u_o.astype(np.float32).astype(np.float64)
+            u = torch.from_numpy(u_o).cuda()
+            u = u.float() if precision else u
+            r = torch.empty_like(u)
+            dg.dg_rhs(p.gpu.ctx, u, r)
+            dg.dg_sync(p.gpu.ctx)
+            got.append(r.double().cpu().numpy())
+            if sf == 0:
+                bar = 16.0 * cases.rounding_floor(p.orc, u_o, eps=2.0 ** (-24 if precision else -53))
+        finally:
+            p.close()
+    err = cases.field_errors(got[1], got[0], 1, 3)
+    print(N, precision, "difference of the routes", err, "bar", bar)
+    assert np.all(err < bar), (err, bar)
