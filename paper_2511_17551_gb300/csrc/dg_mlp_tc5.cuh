@@ -197,8 +197,9 @@ __device__ __forceinline__ float2 gelu2(float2 x) {
 }
 
 // The tile engine (after alloc_tmem and load_weights): for each tile of NR x 128 rows of the CTA, thread t takes
-// the rows tile NR 128 + 128 r + t.  prod(row, x, r) writes the row's 7 standardised features and
-// returns a flag of its own; cons(row, out, flag, valid, r) gets the NO outputs, that flag and
+// the rows tile NR 128 + 128 r + t.  prod(row, x, r, free) writes the row's 7 standardised features and
+// returns a flag of its own (free: no MMA reads the operands, which it may then use for staging; false
+// after a timeout); cons(row, out, flag, valid, r) gets the NO outputs, that flag and
 // whether the launch's tensor-core waits all completed (when not, out is not valid).  Both are
 // called by every thread of the CTA for every tile and r in turn (rows >= n included), so consumers
 // may use warp votes.  The engine frees the tensor memory and returns false
@@ -246,7 +247,7 @@ __device__ __forceinline__ bool run_tiles(Smem<NO, NR>& s, int64_t n, Prod prod,
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
       float x[8];
-      flag[r] = prod(row0 + r * ROWS, x, r);
+      flag[r] = prod(row0 + r * ROWS, x, r, ok);
       // features -> A of layer 1 (this thread's row: K 0-7 and the zero padding 8-15)
       uint4 lo;
       lo.x = dgmlp::pack_bf16(x[0], x[1]);
@@ -254,7 +255,7 @@ __device__ __forceinline__ bool run_tiles(Smem<NO, NR>& s, int64_t n, Prod prod,
       lo.z = dgmlp::pack_bf16(x[4], x[5]);
       lo.w = dgmlp::pack_bf16(x[6], x[7]);
       unsigned char* xb = reinterpret_cast<unsigned char*>(s.X + r * ROWS * 16);
-      if (ok) {  // after a timeout MMAs may still be reading the operands
+      if (ok) {  // after a timeout MMAs may still be reading the operands (X, and H below)
         *reinterpret_cast<uint4*>(xb + canon(tid, 0, 16)) = lo;
         *reinterpret_cast<uint4*>(xb + canon(tid, 8, 16)) = make_uint4(0u, 0u, 0u, 0u);
       }
@@ -379,7 +380,7 @@ __device__ __forceinline__ bool run_tiles(Smem<NO, NR>& s, int64_t n, Prod prod,
 
 // y[n][NO] = network(X[n][7]) for standardised X.  *err is set to 1 when a bounded wait ran
 // out (the outputs of that launch are then not valid).  Launch with THREADS threads and
-// dynamic shared memory of sizeof(Smem<NO>).  A tile's rows are contiguous in X and y: both go
+// dynamic shared memory of sizeof(Smem<NO, FWD_NR>).  A tile's rows are contiguous in X and y: both go
 // through shared memory in 16-byte accesses where the pointers allow (vec), the next tile's
 // X requested while this one is computed; a thread's own row at a time would touch each
 // 32-byte sector up to eight times.
@@ -408,14 +409,14 @@ __global__ void __launch_bounds__(THREADS, FWD_CTAS)
     }
   };
   fetch(blockIdx.x);
-  auto prod = [&](int64_t row, float* x, int r) {
+  auto prod = [&](int64_t row, float* x, int r, bool free) {
     const int64_t tile = row / (NR * ROWS);
     if (vec && (tile + 1) * (NR * ROWS) <= n) {  // the same in all threads
       if (r == 0) {
 #pragma unroll
         for (int j = 0; j < PER; ++j) {
           const int i = tid + j * THREADS;
-          if (i < V4) reinterpret_cast<float4*>(xs)[i] = next[j];
+          if (free && i < V4) reinterpret_cast<float4*>(xs)[i] = next[j];
         }
         fetch(tile + gridDim.x);
         __syncthreads();
