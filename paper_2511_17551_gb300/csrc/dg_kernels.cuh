@@ -42,13 +42,16 @@ struct BasisTab {
 
 template <typename real> struct RealOps;
 // FP64 reciprocal and square root from the hardware's approximations (rcp.approx.ftz.f64 and
-// rsqrt.approx.ftz.f64: relative error about 2^-22) and one cubically convergent step each: with
+// rsqrt.approx.ftz.f64, which look at the upper half of the argument: relative error up to 2^-19.9, measured
+// over FP64's normal numbers) and one cubically convergent step each: with
 // e = 1 - x y the reciprocal is y (1 + e + e^2 + ...), with e = 1 - x y^2 the square root is
 // x y (1 + e/2 + 3 e^2/8 + ...) (Householder's method of order three); what is cut off is below
-// 2^-63.  3 and 5 operations of the FP64 pipe, which bounds the FP64 kernels.  Zeros, infinities
+// 2^-58, and the results are within a unit in the last place of the correctly rounded ones.
+// 3 and 5 operations of the FP64 pipe, which bounds the FP64 kernels.  Zeros, infinities
 // and NaN give what they should by integer tests and selects (a branch to the general functions for
-// them cost more than the operations saved); subnormal arguments count as zeros, subnormal
-// reciprocals are zeros.  FP64 right-hand side of the 32^3 N = 3 Navier-Stokes mesh with __drcp_rn
+// them cost more than the operations saved).  Below FP64's normal numbers: the reciprocal of a
+// subnormal argument is infinite, a subnormal reciprocal is zero, and the square root of a subnormal
+// argument is that argument.  FP64 right-hand side of the 32^3 N = 3 Navier-Stokes mesh with __drcp_rn
 // and sqrt 2534 us, with these 2372 us.
 template <> struct RealOps<double> {
   static __device__ __forceinline__ double rcp(double x) {
