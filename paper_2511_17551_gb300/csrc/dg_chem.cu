@@ -636,7 +636,7 @@ chem_mlp_tc5_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, co
   enter();
   __syncthreads();
   const float dt = dtp ? (float)*dtp : 0.f;
-  auto prod = [&](int64_t i, float* x, int, bool) {
+  auto prod = [&](int64_t i, float* x, int) {
     float raw[7];
     bool ok = true;
     if (i < total) {

@@ -85,7 +85,7 @@ thermo_mlp_kernel(const T* u, int64_t K, int np, int dim, const double* sp, cons
   const int64_t total = K * np;
   unsigned long long n_ok = 0, n_fb = 0;
   double Y[NSPEC], rho = 1.0, e = 0.0;  // this thread's node, carried from features to polish
-  auto prod = [&](int64_t i, float* x, int, bool) {
+  auto prod = [&](int64_t i, float* x, int) {
     if (i < total) {
       const T* uu = u + (i / np) * nv * np + (i % np);
       rho = 0.0;

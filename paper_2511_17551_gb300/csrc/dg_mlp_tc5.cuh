@@ -197,13 +197,13 @@ __device__ __forceinline__ float2 gelu2(float2 x) {
 }
 
 // The tile engine (after alloc_tmem and load_weights): for each tile of NR x 128 rows of the CTA, thread t takes
-// the rows tile NR 128 + 128 r + t.  prod(row, x, r, free) writes the row's 7 standardised features and
-// returns a flag of its own (free: no MMA reads the operands, which it may then use for staging; false
-// after a timeout); cons(row, out, flag, valid, r) gets the NO outputs, that flag and
+// the rows tile NR 128 + 128 r + t.  prod(row, x, r) writes the row's 7 standardised features and
+// returns a flag of its own; cons(row, out, flag, valid, r) gets the NO outputs, that flag and
 // whether the launch's tensor-core waits all completed (when not, out is not valid).  Both are
 // called by every thread of the CTA for every tile and r in turn (rows >= n included), so consumers
 // may use warp votes.  The engine frees the tensor memory and returns false
-// after a timeout (the remaining tiles still reach cons with valid = false).  skip(row of
+// after a timeout (the remaining tiles still reach cons with valid = false, or with STOP are left out:
+// for a prod that stages in the operands, which MMAs may then still be reading).  skip(row of
 // thread t), called by every thread before a tile and returning the same in all, leaves the tile
 // out.  The grid's CTAs from `first` on share the tiles.
 // Tensor memory for the engine, first thing in a kernel (its latency then passes beside the loading
@@ -220,7 +220,7 @@ __device__ __forceinline__ void alloc_tmem(Smem<NO, NR>& s) {
 struct NoSkip {
   __device__ __forceinline__ bool operator()(int64_t) const { return false; }
 };
-template <int NO, int NR, class Prod, class Cons, class Skip = NoSkip>
+template <int NO, int NR, bool STOP = false, class Prod, class Cons, class Skip = NoSkip>
 __device__ __forceinline__ bool run_tiles(Smem<NO, NR>& s, int64_t n, Prod prod, Cons cons, Skip skip = Skip(),
                                           int first = 0) {
   constexpr int NH = DG_MLP_NH;
@@ -247,7 +247,7 @@ __device__ __forceinline__ bool run_tiles(Smem<NO, NR>& s, int64_t n, Prod prod,
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
       float x[8];
-      flag[r] = prod(row0 + r * ROWS, x, r, ok);
+      flag[r] = prod(row0 + r * ROWS, x, r);
       // features -> A of layer 1 (this thread's row: K 0-7 and the zero padding 8-15)
       uint4 lo;
       lo.x = dgmlp::pack_bf16(x[0], x[1]);
@@ -364,6 +364,7 @@ __device__ __forceinline__ bool run_tiles(Smem<NO, NR>& s, int64_t n, Prod prod,
       for (int o = 0; o < NO; ++o) out[o] = acc[r][o].x + acc[r][o].y;
       cons(row0 + r * ROWS, out, flag[r], ok, r);
     }
+    if (STOP && !ok) break;
     fence_before();
     __syncthreads();  // the next tile rewrites X, H and the accumulators
     fence_after();
@@ -409,14 +410,14 @@ __global__ void __launch_bounds__(THREADS, FWD_CTAS)
     }
   };
   fetch(blockIdx.x);
-  auto prod = [&](int64_t row, float* x, int r, bool free) {
+  auto prod = [&](int64_t row, float* x, int r) {
     const int64_t tile = row / (NR * ROWS);
     if (vec && (tile + 1) * (NR * ROWS) <= n) {  // the same in all threads
       if (r == 0) {
 #pragma unroll
         for (int j = 0; j < PER; ++j) {
           const int i = tid + j * THREADS;
-          if (free && i < V4) reinterpret_cast<float4*>(xs)[i] = next[j];
+          if (i < V4) reinterpret_cast<float4*>(xs)[i] = next[j];
         }
         fetch(tile + gridDim.x);
         __syncthreads();
@@ -445,7 +446,7 @@ __global__ void __launch_bounds__(THREADS, FWD_CTAS)
       for (int o = 0; o < NO; ++o) y[row * NO + o] = out[o];
     }
   };
-  if (!run_tiles<NO, NR>(s, n, prod, cons) && threadIdx.x == 0) atomicExch(err, 1u);
+  if (!run_tiles<NO, NR, true>(s, n, prod, cons) && threadIdx.x == 0) atomicExch(err, 1u);
 }
 
 }  // namespace dgtc5
