@@ -765,7 +765,9 @@ chem_fallback_kernel(const T* u, const double* Tc, int64_t K, int np, int dim, c
   const int nv = NSPEC + dim + 1;
   const int lane = threadIdx.x & 31;
   const int64_t total = K * np, ntiles = (total + 31) / 32;
-  const T tol = (T)mlp->tol_check, floor_ = (T)mlp->floor;
+  // (a tolerance above the form's range stays finite: infinity times a zero scale accepts nothing)
+  const T tol = (T)fmin(mlp->tol_check, sizeof(T) == 4 ? 3.4028234663852886e38 : 1.7976931348623157e308);
+  const T floor_ = (T)mlp->floor;
   typename ChemForm<T>::step dt;
   form_step(dtp ? *dtp : 0.0, dt);
   unsigned long long n_ok = 0, n_fb = 0;
