@@ -35,5 +35,7 @@ inline cudaError_t launch_pdl(bool apart, void (*k)(P...), unsigned grid, unsign
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = apart ? 0 : 1;
-  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(a)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k, static_cast<P>(a)...);
+  if (e != cudaSuccess) cudaGetLastError();  // reported here: not to the next call that asks
+  return e;
 }
