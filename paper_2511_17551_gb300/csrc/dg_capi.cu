@@ -942,6 +942,8 @@ dg_status dg_init_mesh(const dg_mesh_desc* m, const dg_physics_desc* p, dg_ctx**
       cudaFree(bw);
       TRY(e2);
     }
+    // (needed: the first kernels of the context read the metric terms without waiting for the kernels
+    // before them, own_metrics)
     TRY(cudaStreamSynchronize(c->stream));
   }
   free(nbr_h);

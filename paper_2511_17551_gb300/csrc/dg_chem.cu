@@ -414,7 +414,8 @@ __device__ __noinline__ void chem_node_general(const float* uu, int np, double T
 
 // The plain source of one node in the two forms: the rates in the form's arithmetic, and
 // S_s = omega_s / (1 + dt jpi_s) rounded to the form.  Every kernel that evaluates the plain
-// source goes through these, so that they agree bit for bit.
+// source for a step goes through these, so that they agree bit for bit (the training samples of
+// chem_sample_kernel are FP64 in both forms).
 struct Chem64 {  // FP64 form
   struct Tab {};
   struct Args {};  // the pairs' table is no argument of this form's kernels

@@ -40,7 +40,7 @@ struct DgArgs {
                           // CTAs still read their neighbours' input low parts)
   const void* Ja;         // [K][dim][dim][np]
   const void* invJ;       // [K][np]
-  int own_metrics;        // Ja and invJ are a context's, written once when it was made
+  int own_metrics;        // Ja and invJ are a context's: written when it was made, and no kernel of that is in flight
   int apart;              // kernels start one after the other (per-kernel timing)
   void* gradW;            // [K][dim][dim+1][np] (Navier-Stokes): grad_mode 0 the contravariant
                           // viscous fluxes [d][c] = sum_x Ja^d_x f^v_{x,c}; 1 the gradients [x][c]

@@ -8,8 +8,8 @@
 //
 // The time steps are chains of kernels of 10 to 200 us, each of which used to wait for the last
 // CTA of the one before, its memory flush and its own launch.  10 steps of the 12 x 10 x 9 N = 4
-// Navier-Stokes mesh: 1394 -> 1163 us; 32^3 N = 3: 8.89 -> 8.55 ms; five of the 131 k element cylinder:
-// 3.24 -> 3.10 ms; meshes of a few elements: 15 to 30 % less.  The trigger of the two long
+// Navier-Stokes mesh: 1394 -> 1122 us; 32^3 N = 3: 8.89 -> 8.51 ms; five of the 131 k element cylinder:
+// 3.24 -> 3.09 ms (each with the state set and read back); meshes of a few elements: 15 to 30 % less.  The trigger of the two long
 // kernels (right-hand side, gradients) stands before their last phase: at their start it cost 3 to
 // 14 % against there, since the next kernel's CTAs then take the places that their own CTAs leave
 // and lie unevenly on the SMs.  In FP64, where the FP64 pipe of an SM bounds its CTAs, that weighs

@@ -428,8 +428,8 @@ rhs_kernel(const DgArgs a, const KConst kc) {
           bulk_g2s(dst + e * sstride, src + (e0 + e) * block, (unsigned)(RS * block), &s_bar);
         }
       };
-      // the context's metric terms are no kernel's output: requested before the preceding
-      // kernel has ended (a caller's own arrays may be)
+      // a context's metric terms are written only while it is made, which ends in a synchronisation:
+      // requested before the preceding kernel has ended (a caller's own arrays may be its output)
       if (!a.own_metrics) pdl_wait();
       for (int j = tid; j < 2 * ne; j += 32) {
         if (j & 1) copy(sja, L::SJA, (const real*)a.Ja, DIM * DIM * NP, j >> 1);
