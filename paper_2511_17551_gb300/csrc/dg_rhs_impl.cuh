@@ -1280,8 +1280,10 @@ __global__ void __launch_bounds__(128) positivity_kernel(const DgArgs a, real* u
   const int64_t k0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * EPW;
   // The next kernel's CTAs: behind the screening, since resident early they leave the right-hand side
   // after them unevenly placed (N = 2, 20^3 elements with indicator and limiter, four steps: 749 against 1,163 us;
-  // 14^3, N = 3: 585 against 672); at once where the grid leaves most SMs free (10^3, N = 2: 546 against 564)
-  const bool early = gridDim.x <= 64;
+  // 14^3, N = 3: 585 against 672).  At once where the grid leaves most SMs free (10^3, N = 2: 546 against 564),
+  // and for mixtures, where the temperature solve comes between (400 elements, N = 4, three steps: 375
+  // against 425 us; 5,760, N = 3: 925 against 934)
+  const bool early = NSP > 1 || gridDim.x <= 64;
   if (early) trigger();
   if (k0 >= a.K) return;  // uniform per warp
   const int ch = (int)((a.K - k0) < EPW ? (a.K - k0) : EPW) * NP;
